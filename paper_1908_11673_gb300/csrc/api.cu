@@ -294,6 +294,10 @@ int qxd_apply_Dw(qxd_ctx* ctx, int fl, int prec, const void* in, void* out, int 
     bool host_out;
     QXD_TRY(stage_in(ctx, WS_STAGE_IN, in, cbytes, &din, st));
     QXD_TRY(stage_out(ctx, WS_STAGE_OUT, out, cbytes, &dout, &host_out));
+    if (prec != QXD_DF64 && canon_fits(din, dout, cbytes, false)) {
+        QXD_TRY(op_Dw_canon(ctx, fl, prec, din, dout, nrhs, st));
+        return finish_out(ctx, out, dout, cbytes, host_out, st);
+    }
     const size_t hb = half_bytes(ctx, prec) * nrhs;
     void *ie, *io, *oe, *oo;
     QXD_TRY(qxd_ws(ctx, WS_T0, hb, &ie));
@@ -334,8 +338,12 @@ int qxd_apply_Dhat_eo(qxd_ctx* ctx, int fl, int prec, int dagger, const void* in
     QXD_TRY(stage_out(ctx, WS_STAGE_OUT, out_e, cbytes, &dout, &host_out));
     const size_t hb = half_bytes(ctx, prec) * nrhs;
     void *ie, *to, *oe;
-    QXD_TRY(qxd_ws(ctx, WS_T0, hb, &ie));
     QXD_TRY(qxd_ws(ctx, WS_T1, hb, &to));
+    if (canon_fits(din, dout, cbytes, true)) {
+        QXD_TRY(op_Dhat_canon(ctx, fl, prec, dagger ? 1 : 0, din, dout, to, nrhs, st));
+        return finish_out(ctx, out_e, dout, cbytes, host_out, st);
+    }
+    QXD_TRY(qxd_ws(ctx, WS_T0, hb, &ie));
     QXD_TRY(qxd_ws(ctx, WS_T2, hb, &oe));
     QXD_TRY(launch_pack(ctx, cprec, din, 0, 0, prec, ie, nrhs, st));
     QXD_TRY(op_Dhat(ctx, fl, prec, dagger ? 1 : 0, ie, oe, to, st, nrhs));

@@ -29,6 +29,13 @@ int op_Dhat(qxd_ctx* ctx, int fl, int P, int dagger, const void* in_e, void* out
 int op_Dhat_dots(qxd_ctx* ctx, int fl, const void* in_e, void* out_e, void* tmp_o, int k, const void* const* W,
                  int slot, cudaStream_t st);
 int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* const* W, int slot, cudaStream_t st);
+// The same operators on the caller's canonical fields (hop_canon.cu; FP64, FP32, BF16
+// storage), where canon_fits(in, out, bytes, in_place) holds: both fields 32-byte aligned
+// and disjoint, or (in_place) one and the same.  tmp_o: internal odd scratch.
+bool canon_fits(const void* in, const void* out, size_t bytes, bool in_place);
+int op_Dw_canon(qxd_ctx* ctx, int fl, int P, const void* in, void* out, int nrhs, cudaStream_t st);
+int op_Dhat_canon(qxd_ctx* ctx, int fl, int P, int dagger, const void* in_e, void* out_e, void* tmp_o, int nrhs,
+                  cudaStream_t st);
 // b_e = r_e - H_eo A_oo^-1 r_o  (even-odd preconditioned source)
 int op_eo_source(qxd_ctx* ctx, int fl, int P, const Full& r, void* b_e, void* tmp_o, cudaStream_t st, int nrhs = 1);
 // x_o = A_oo^-1 (r_o - H_oe x_e)
