@@ -139,17 +139,29 @@ __device__ __forceinline__ void canon_hop(const Geo& g, const CanonDev& a, const
     reconstruct<MU, FWD>(r, acc);
 }
 
-// Block (S, R): S consecutive sites of R right-hand sides, so that the links and diagonal
-// terms that the first of them brings into L1 serve the others; block b covers the
-// right-hand-side group b % ngroups of the site tile b / ngroups.
+// One thread per site and right-hand side, one warp per block; block b covers right-hand
+// side b % nrhs of the site tile b / nrhs, so that the links and diagonal terms that the
+// first of them brings into L2 serve the others.
+//
+// Latency-bound: what counts is loads in flight per thread, not warps.  The launch bound
+// names 256 threads although a block has 32: with it the compiler spends 146 to 165
+// registers (12 warps per SM) and starts several directions' loads early; with bounds
+// that let it use 96 to 128 the same kernel is slower, as is an explicit prefetch of the
+// next direction, two or four right-hand sides per thread (one link load for all), or
+// blocks that hold four right-hand sides.  Measured (us; blocks of 4 right-hand sides or
+// 128 sites -> here): D_w 24^3x48, 12 right-hand sides 1102 -> 761, Dhat^+ 24^3x48 126 ->
+// 104, Dhat 32^3x64 C* 685 -> 585 (1952 bytes per even site at 7.0 TB/s).  With many
+// right-hand sides the L1 data pipe is 76 % busy: a 96-byte stride takes two passes per
+// 256-bit load where the internal layout takes one.
+constexpr int kCanonThreads = 32;
+
 template <int P, int MODE>
-__global__ void __launch_bounds__(256) k_hop_canon(Geo g, CanonDev a, int nrhs, int ngroups) {
+__global__ void __launch_bounds__(256, 1) k_hop_canon(Geo g, CanonDev a, int nrhs) {
     using R = typename Prec<P>::real;
-    const int grp = blockIdx.x % ngroups;
-    const int i = (blockIdx.x / ngroups) * blockDim.x + threadIdx.x;
-    const int rhs = grp * blockDim.y + threadIdx.y;
+    const int rhs = blockIdx.x % nrhs;
+    const int i = (blockIdx.x / nrhs) * kCanonThreads + threadIdx.x;
     const int Vh = g.Vh;
-    if (i >= (MODE == kDw ? (int)g.V : Vh) || rhs >= nrhs) return;
+    if (i >= (MODE == kDw ? (int)g.V : Vh)) return;
     int x[4], p, h;
     if constexpr (MODE == kDw) {
         int r = i;
@@ -231,15 +243,10 @@ int launch_canon(qxd_ctx* ctx, int fl, int prec, const void* nb, const void* sel
     std::snprintf(name, sizeof name, "hop_%s_%s%s", prec == QXD_FP64 ? "fp64" : prec == QXD_FP32 ? "fp32" : "bf16", mode,
                   nrhs > 1 ? "_mrhs" : "");
     ProfScope prof(ctx, name, (double)g.Vh * ((MODE == kDw ? link + 2 * dg : link + dg) + per * nrhs), st);
-    const int R = nrhs < 4 ? nrhs : 4;
-    const int S = nrhs == 1 ? 128 : 64;
-    const int ngroups = (nrhs + R - 1) / R;
-    const long long sites = MODE == kDw ? g.V : g.Vh;
-    const unsigned grid = (unsigned)(nblocks(sites, S) * ngroups);
-    const dim3 blk(S, R);
-    if (prec == QXD_FP64) k_hop_canon<0, MODE><<<grid, blk, 0, st>>>(g, a, nrhs, ngroups);
-    else if (prec == QXD_FP32) k_hop_canon<1, MODE><<<grid, blk, 0, st>>>(g, a, nrhs, ngroups);
-    else k_hop_canon<2, MODE><<<grid, blk, 0, st>>>(g, a, nrhs, ngroups);
+    const int grid = nblocks(MODE == kDw ? g.V : g.Vh, kCanonThreads) * nrhs;
+    if (prec == QXD_FP64) k_hop_canon<0, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs);
+    else if (prec == QXD_FP32) k_hop_canon<1, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs);
+    else k_hop_canon<2, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs);
     QXD_CUDA(ctx, cudaGetLastError());
     return QXD_OK;
 }
