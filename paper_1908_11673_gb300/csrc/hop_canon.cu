@@ -2,7 +2,7 @@
 // ([site][4][3] complex, Sec. 2.3 operator), without a pass that converts them to
 // the internal structure-of-arrays layout and back.
 //
-//   kDw     out = D in on the full lattice, both parities in one launch
+//   kDw     out = D in on the full lattice, both parities in the same launch
 //   kDhat1  t_o = A_oo^-1 H_oe in_e, canonical even field in, internal odd field out
 //   kDhat2  out_e = A_ee in_e - H_eo t_o, internal odd field and canonical even field in,
 //           canonical even field out
@@ -156,12 +156,12 @@ __device__ __forceinline__ void canon_hop(const Geo& g, const CanonDev& a, const
 constexpr int kCanonThreads = 32;
 
 template <int P, int MODE>
-__global__ void __launch_bounds__(256, 1) k_hop_canon(Geo g, CanonDev a, int nrhs) {
+__global__ void __launch_bounds__(256, 1) k_hop_canon(Geo g, CanonDev a, int nrhs, int first, int end) {
     using R = typename Prec<P>::real;
     const int rhs = blockIdx.x % nrhs;
-    const int i = (blockIdx.x / nrhs) * kCanonThreads + threadIdx.x;
+    const int i = first + (blockIdx.x / nrhs) * kCanonThreads + threadIdx.x;
     const int Vh = g.Vh;
-    if (i >= (MODE == kDw ? (int)g.V : Vh)) return;
+    if (i >= end) return;
     int x[4], p, h;
     if constexpr (MODE == kDw) {
         int r = i;
@@ -242,12 +242,19 @@ int launch_canon(qxd_ctx* ctx, int fl, int prec, const void* nb, const void* sel
     char name[48];
     std::snprintf(name, sizeof name, "hop_%s_%s%s", prec == QXD_FP64 ? "fp64" : prec == QXD_FP32 ? "fp32" : "bf16", mode,
                   nrhs > 1 ? "_mrhs" : "");
-    ProfScope prof(ctx, name, (double)g.Vh * ((MODE == kDw ? link + 2 * dg : link + dg) + per * nrhs), st);
-    const int grid = nblocks(MODE == kDw ? g.V : g.Vh, kCanonThreads) * nrhs;
-    if (prec == QXD_FP64) k_hop_canon<0, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs);
-    else if (prec == QXD_FP32) k_hop_canon<1, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs);
-    else k_hop_canon<2, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs);
-    QXD_CUDA(ctx, cudaGetLastError());
+    // D_w of several right-hand sides goes over the sites in two launches (the first and the
+    // second half), as many as the half-lattice kernels take; one right-hand side in one
+    const int sites = MODE == kDw ? (int)g.V : g.Vh;
+    const int parts = MODE == kDw && nrhs > 1 ? 2 : 1;
+    for (int k = 0; k < parts; ++k) {
+        const int first = k * (sites / parts), end = k + 1 == parts ? sites : (k + 1) * (sites / parts);
+        ProfScope prof(ctx, name, (double)g.Vh * ((MODE == kDw ? link + 2 * dg : link + dg) + per * nrhs) / parts, st);
+        const int grid = nblocks(end - first, kCanonThreads) * nrhs;
+        if (prec == QXD_FP64) k_hop_canon<0, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs, first, end);
+        else if (prec == QXD_FP32) k_hop_canon<1, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs, first, end);
+        else k_hop_canon<2, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs, first, end);
+        QXD_CUDA(ctx, cudaGetLastError());
+    }
     return QXD_OK;
 }
 
