@@ -10,9 +10,35 @@
 
 using namespace qxd;
 
+static void free_fields(QxdFlavour& F) {
+    cudaFree(F.V64);
+    cudaFree(F.Z32);
+    F.V64 = nullptr;
+    F.Z32 = nullptr;
+    for (int k = 0; k < 2; ++k) {
+        cudaFree(F.C64[k]);
+        cudaFree(F.C32[k]);
+        F.C64[k] = nullptr;
+        F.C32[k] = nullptr;
+    }
+}
+
 int qxd_fail(qxd_ctx* ctx, int code, const std::string& msg) {
     if (ctx) ctx->err = msg;
     return code;
+}
+
+// Device memory of `bytes` bytes; when there is none left, the field buffers that
+// qxd_set_links kept for flavours not set again since are given back first.
+bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes) {
+    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    for (auto& F : ctx->fl)
+        if (!F.set && !F.building) free_fields(F);
+    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    *p = nullptr;
+    return false;
 }
 
 int qxd_ws(qxd_ctx* ctx, int slot, size_t bytes, void** out) {
@@ -26,8 +52,7 @@ int qxd_ws(qxd_ctx* ctx, int slot, size_t bytes, void** out) {
         ctx->ws_ptr[slot] = nullptr;
         ctx->ws_size[slot] = 0;
         void* p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess) {
-            cudaGetLastError();
+        if (!dev_alloc(ctx, &p, bytes)) {
             return qxd_fail(ctx, QXD_ENOMEM, "workspace allocation of " + std::to_string(bytes) + " bytes failed");
         }
         ctx->ws_ptr[slot] = p;
@@ -154,21 +179,29 @@ bool make_geo(const qxd_geom* g, Geo* G) {
     return true;
 }
 
-static void free_flavour(QxdFlavour& F) {
-    cudaFree(F.V64);
-    cudaFree(F.Z32);
-    for (int k = 0; k < 2; ++k) {
-        cudaFree(F.C64[k]);
-        cudaFree(F.C32[k]);
-        cudaFree(F.Cdf[k]);
-    }
+// drops everything a flavour holds but its field buffers, which qxd_set_clover fills again
+static void reset_flavour(QxdFlavour& F) {
+    cudaFree(F.Cdf[0]);
+    cudaFree(F.Cdf[1]);
     cudaFree(F.Vdf);
     cudaFree(F.W);
     cudaFree(F.dfl_basis);
     cudaFree(F.dfl_A);
     cudaFree(F.dfl_nbr);
     cudaFree(F.dfl_stat);
-    F = QxdFlavour{};
+    QxdFlavour kept{};
+    kept.V64 = F.V64;
+    kept.Z32 = F.Z32;
+    for (int k = 0; k < 2; ++k) {
+        kept.C64[k] = F.C64[k];
+        kept.C32[k] = F.C32[k];
+    }
+    F = kept;
+}
+
+static void free_flavour(QxdFlavour& F) {
+    reset_flavour(F);
+    free_fields(F);
 }
 
 extern "C" {
@@ -237,7 +270,7 @@ int qxd_set_links(qxd_ctx* ctx, const double* U, const double* A, double invqel,
     const void *dU, *dA;
     QXD_TRY(stage_in(ctx, WS_STAGE_U, U, Vp * 4 * 9 * 16, &dU, st));
     QXD_TRY(stage_in(ctx, WS_STAGE_A, A, Vp * 4 * 8, &dA, st));
-    for (auto& F : ctx->fl) free_flavour(F);
+    for (auto& F : ctx->fl) reset_flavour(F);
     QXD_TRY(launch_set_links(ctx, static_cast<const double2*>(dU), static_cast<const double*>(dA), st));
     QXD_CUDA(ctx, cudaStreamSynchronize(st));
     ctx->links_set = true;
@@ -253,21 +286,18 @@ int qxd_set_clover(qxd_ctx* ctx, int fl, const qxd_flavour* f, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     QxdFlavour& F = ctx->fl[fl];
     const size_t Vh = ctx->g.Vh;
+    F.set = false;
+    F.building = true;  // its buffers are not spare
     if (!F.V64) {
-        bool ok = cudaMalloc(&F.V64, 2 * 36 * Vh * sizeof(double2)) == cudaSuccess &&
-                  cudaMalloc(&F.Z32, 2 * 2 * Vh * sizeof(float4)) == cudaSuccess &&
-                  cudaMalloc(&F.C64[0], 2 * 36 * Vh * sizeof(double2)) == cudaSuccess &&
-                  cudaMalloc(&F.C64[1], 2 * 36 * Vh * sizeof(double2)) == cudaSuccess &&
-                  cudaMalloc(&F.C32[0], 2 * 18 * Vh * sizeof(float4)) == cudaSuccess &&
-                  cudaMalloc(&F.C32[1], 2 * 18 * Vh * sizeof(float4)) == cudaSuccess;
+        auto get = [&](auto** p, size_t n) { return dev_alloc(ctx, reinterpret_cast<void**>(p), n * sizeof(**p)); };
+        bool ok = get(&F.V64, 2 * 36 * Vh) && get(&F.Z32, 2 * 2 * Vh) && get(&F.C64[0], 2 * 36 * Vh) &&
+                  get(&F.C64[1], 2 * 36 * Vh) && get(&F.C32[0], 2 * 18 * Vh) && get(&F.C32[1], 2 * 18 * Vh);
         if (!ok) {
-            cudaGetLastError();
             free_flavour(F);
             return qxd_fail(ctx, QXD_ENOMEM, "set_clover: allocation failed");
         }
     }
     F.f = *f;
-    F.set = false;
     // double-float copies and a deflation subspace belong to the operator they were built for
     cudaFree(F.Vdf);
     cudaFree(F.Cdf[0]);
@@ -275,9 +305,10 @@ int qxd_set_clover(qxd_ctx* ctx, int fl, const qxd_flavour* f, void* stream) {
     F.Vdf = nullptr;
     F.Cdf[0] = F.Cdf[1] = nullptr;
     dfl_free(F);
-    QXD_TRY(launch_set_flavour(ctx, fl, st));
-    F.set = true;
-    return QXD_OK;
+    const int rc = launch_set_flavour(ctx, fl, st);
+    F.building = false;
+    F.set = rc == QXD_OK;
+    return rc;
 }
 
 int qxd_apply_Dw(qxd_ctx* ctx, int fl, int prec, const void* in, void* out, int nrhs, void* stream) {

@@ -15,6 +15,7 @@
 
 struct QxdFlavour {
     bool set = false;
+    bool building = false;  // inside qxd_set_clover
     qxd_flavour f{};
     double2* V64 = nullptr;    // [p][36][Vh]   V = U z^qhat (boundary phase folded in)
     float4* Z32 = nullptr;     // [p][2][Vh]    z^qhat (boundary phase folded in)
@@ -109,6 +110,9 @@ int qxd_fail(qxd_ctx* ctx, int code, const std::string& msg);
 // workspace slot `slot` with at least `bytes` bytes (device memory)
 int qxd_ws(qxd_ctx* ctx, int slot, size_t bytes, void** out);
 
+// device memory for the context (api.cu); false if there is none
+bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes);
+
 // caller arrays at the C ABI (api.cu): a device view of an input (the array
 // itself when it is device memory, else a copy staged in workspace `slot`); a
 // device destination for an output and whether it must be copied back to the
@@ -129,6 +133,7 @@ enum {
     WS_SAP = 272,
     WS_RAT = 288,
     WS_DFL = 300,
+    WS_CLOVER = 318,
     WS_NSLOTS = 320
 };
 
