@@ -73,257 +73,458 @@ QXD_HD void link_for(const Geo& g, const PtcLinks& L, int d, int p, int h, const
     else load_link32(L.U32 + (size_t)ps * 12 * Vh, L.Z32 + (size_t)ps * 2 * Vh, Vh, mu, lk.src, lk.m, lk.z);
 }
 
-template <int I>
-QXD_HD void transport_row(const Geo& g, int d, int p, int h, const PtcLink& lk, const float4* __restrict__ a_ch,
-                          cplx<float> t[4]) {
-    const int Vh = g.Vh;
-    if (d == 0) {
-        const float4* b = a_ch + (size_t)p * 6 * Vh;
+// two FP32 multiply-adds (products) in one instruction
+__device__ __forceinline__ unsigned long long f2_bits(float2 a) { return *reinterpret_cast<unsigned long long*>(&a); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+    return *reinterpret_cast<float2*>(&d);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return *reinterpret_cast<float2*>(&d);
+}
+
+// the link of direction d > 0 with its phase, V = U z^qhat
+__device__ __forceinline__ void vlink_for(const Geo& g, const PtcLinks& L, int d, int p, int h, const int x[4],
+                                          Mat3<float>& V, int& src) {
+    PtcLink lk;
+    link_for(g, L, d, p, h, x, lk);
+    src = lk.src;
 #pragma unroll
-        for (int sp = 0; sp < 4; ++sp) {
-            const int q = 3 * sp + I;
-            const float4 v = QXD_LDG(b + (size_t)(q >> 1) * Vh + h);
-            t[sp] = (q & 1) ? cplx<float>{v.z, v.w} : cplx<float>{v.x, v.y};
-        }
-        return;
-    }
-    cplx<float> s[12];
-    load_spinor<1>(a_ch + (size_t)(1 - p) * 6 * Vh, Vh, lk.src, s);
-    const bool fwd = d <= 4;
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int sp = 0; sp < 4; ++sp) {
-        cplx<float> acc = {0.f, 0.f};
+        for (int j = 0; j < 3; ++j) V.a[i][j] = lk.z * lk.m.a[i][j];
+}
+
+// t = V s (forwards) or V^+ s on the colours of a spinor.  Scalar FP32 instructions run at
+// half the rate of the packed ones on this GPU (39 against 67 TFLOP/s measured): a packed
+// multiply-add takes the real or the imaginary part of an entry times a complex number.
+__device__ __forceinline__ void transport_v(const Mat3<float>& V, bool fwd, const cplx<float> s[12],
+                                            cplx<float> t[12]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float2 A[4], B[4];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            if (fwd) cmac(acc, lk.m.a[I][j], s[3 * sp + j]);
-            else cmac_conj(acc, lk.m.a[j][I], s[3 * sp + j]);
+            const cplx<float> e = fwd ? V.a[i][j] : V.a[j][i];
+            const float2 er = make_float2(e.re, e.re), ei = make_float2(e.im, e.im);
+#pragma unroll
+            for (int sp = 0; sp < 4; ++sp) {
+                const float2 v = make_float2(s[3 * sp + j].re, s[3 * sp + j].im);
+                A[sp] = j == 0 ? mul2(er, v) : fma2(er, v, A[sp]);
+                B[sp] = j == 0 ? mul2(ei, v) : fma2(ei, v, B[sp]);
+            }
         }
-        t[sp] = fwd ? lk.z * acc : cmul_conj(lk.z, acc);
+#pragma unroll
+        for (int sp = 0; sp < 4; ++sp)
+            t[3 * sp + i] = fwd ? cplx<float>{A[sp].x - B[sp].y, A[sp].y + B[sp].x}
+                                : cplx<float>{A[sp].x + B[sp].y, A[sp].y - B[sp].x};
     }
 }
 
-// ---- forward layer ------------------------------------------------------------------
-// Thread (site, colour I): a tile of kPtcSites sites of one parity, the three
-// colour rows in three groups of kPtcSites threads (warp-uniform colour).  Each
-// thread forms T_d a_{c'} once per (d, c') and accumulates all COUT output
-// channels of its group from it; the group's weights [9][cin][COUT][4][4] sit in
-// shared memory (read as broadcasts).  Persistent: a block loops over tiles.
-constexpr int kPtcSites = 64;
-constexpr int kPtcFwdThreads = 3 * kPtcSites;
-constexpr int kPtcGroup = 8;  // output channels per block (grid.z splits larger layers)
+// What is known to vanish or not to be needed: the network's input, and the adjoint of its
+// last layer, live on the even sites; only even sites of its output are used.
+struct PtcParity {
+    bool in_even;   // input zero on odd sites: even outputs take T_0 only, odd ones T_1 .. T_8
+    bool out_even;  // only even output sites wanted
+};
 
-template <int I, int COUT>
-__device__ void ptc_fwd_site(const Geo& g, const PtcLinks& L, const float4* __restrict__ a, int cin, int ng,
-                             const float2* __restrict__ wsh, float4* __restrict__ out, int c0, int p, int h) {
+// ---- forward layer ------------------------------------------------------------------
+// Per colour a layer is the complex product of the (c, s) x (d, c', s') weights with the
+// transports.  A CTA takes 64 sites of one parity and goes over the 9 cin pairs (d, c') eight
+// at a time: its threads form the transports of eight pairs (a thread one site and two
+// pairs) in shared memory, then every thread multiplies: one site, all colours, NC output
+// channels, the eight warps split over two site groups, CG channel groups and KG groups of
+// the pairs (whose sums are added at the end, in a fixed order).
+//
+// Bound by the FP32 pipe: 27,648 complex multiply-adds per site for 8 -> 8 channels, 194 us
+// on 16^4.  Two spin rows share a packed FP32 instruction; weights are read as broadcasts
+// of whole rows (real, imaginary and negated imaginary planes, so that no sign is formed in
+// the loop), each transport is loaded once per 8 rows.  One thread per (site, colour row)
+// with scalar arithmetic (every transport formed three times, weights re-read per row) took
+// 647 us for 8 -> 8 channels on 16^4; here 424 us (39 us for
+// 1 -> 8 channels, 86 us for 8 -> 1 with even outputs only; 133 us both before). 46 % of the
+// issue slots: what is left besides the products is the staging of the transports, which the
+// two resident CTAs overlap only in part.
+constexpr int kPtcSites = 64;
+constexpr int kPtcThreads = 256;
+constexpr int kPtcPairs = 8;   // (d, c') pairs of a stage
+constexpr int kPtcGroup = 8;   // output channels per block (grid.z splits larger layers)
+
+struct PtcFwdShared {
+    float2 t[4 * kPtcPairs][3][kPtcSites];
+    float w[3][4 * kPtcPairs][4 * kPtcGroup];  // Re W, Im W, -Im W
+};
+
+// weight planes of a layer cin -> cout (adjoint: of the adjoint of the layer cout -> cin with
+// the weights W, W'[c][c'][d] = W[c'][c][opposite(d)]^+): [group of 8 output channels]
+// [pair q = d cin + c'][Re, Im, -Im][s'][4 (c - c0) + s], zero beyond cout
+constexpr int kPlane = 3 * 4 * 4 * kPtcGroup;  // floats of a pair
+
+__global__ void k_ptc_planes(const float2* __restrict__ W, int cin, int cout, int adjoint, float* __restrict__ P) {
+    const int np = 9 * cin, n = ((cout + kPtcGroup - 1) / kPtcGroup) * np * 4 * 4 * kPtcGroup;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        const int row = e % (4 * kPtcGroup), si = (e / (4 * kPtcGroup)) & 3, q = (e / (16 * kPtcGroup)) % np;
+        const int z = e / (16 * kPtcGroup * np);
+        const int c = kPtcGroup * z + row / 4, so = row & 3, d = q / cin, cp = q % cin;
+        float2 v = make_float2(0.f, 0.f);
+        if (c < cout) {
+            const int dop = d == 0 ? 0 : (d <= 4 ? d + 4 : d - 4);
+            v = adjoint ? W[((size_t)(cp * cout + c) * 9 + dop) * 16 + 4 * si + so]
+                        : W[((size_t)(c * cin + cp) * 9 + d) * 16 + 4 * so + si];
+            if (adjoint) v.y = -v.y;
+        }
+        float* o = P + ((size_t)z * np + q) * kPlane + si * 4 * kPtcGroup + row;
+        o[0] = v.x;
+        o[16 * kPtcGroup] = v.y;
+        o[32 * kPtcGroup] = -v.y;
+    }
+}
+
+template <int NC, int CG, int KG>
+__global__ void __launch_bounds__(kPtcThreads, 2) k_ptc_fwd(Geo g, PtcLinks L, const float4* __restrict__ a, int cin,
+                                                           int cout, const float* __restrict__ planes,
+                                                           float4* __restrict__ out, PtcParity par) {
+    static_assert(CG * KG == 4, "eight warps: two site groups, CG channel and KG pair groups");
+    extern __shared__ float4 ptc_sh[];
+    PtcFwdShared& S = *reinterpret_cast<PtcFwdShared*>(ptc_sh);
+    constexpr int R = 4 * NC;       // rows of a thread
+    const int c0 = blockIdx.z * kPtcGroup;
+    const int ng = min(kPtcGroup, cout - c0);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int sg = warp & 1, cg = (warp >> 1) % CG, kg = (warp >> 1) / CG;
+    const int site = 32 * sg + lane;
+    const int st_site = tid & (kPtcSites - 1), st_slot = tid / kPtcSites;
     const size_t chs = (size_t)12 * g.Vh;  // float4 per channel
-    int x[4];
-    site_coords(g, p, h, x);
-    cplx<float> acc[COUT][4];
+    const int tiles = (g.Vh + kPtcSites - 1) / kPtcSites;
+    for (int tile = blockIdx.x; tile < (par.out_even ? tiles : 2 * tiles); tile += gridDim.x) {
+        const int p = tile / tiles;
+        const int h0 = (tile % tiles) * kPtcSites;
+        const int q0 = par.in_even && p == 1 ? cin : 0;
+        const int q1 = par.in_even && p == 0 ? cin : 9 * cin;
+        float2 re[R / 2][3], im[R / 2][3];
 #pragma unroll
-    for (int c = 0; c < COUT; ++c)
+        for (int r = 0; r < R / 2; ++r)
 #pragma unroll
-        for (int sp = 0; sp < 4; ++sp) acc[c][sp] = {0.f, 0.f};
-    for (int d = 0; d < 9; ++d) {
-        PtcLink lk;
-        if (d > 0) link_for(g, L, d, p, h, x, lk);
-        for (int cp = 0; cp < cin; ++cp) {
-            cplx<float> t[4];
-            transport_row<I>(g, d, p, h, lk, a + cp * chs, t);
-            const float4* w = reinterpret_cast<const float4*>(wsh + (size_t)(d * cin + cp) * COUT * 16);
+            for (int i = 0; i < 3; ++i) re[r][i] = im[r][i] = make_float2(0.f, 0.f);
+        const int hs = h0 + st_site;
+        int x[4];
+        if (hs < g.Vh) site_coords(g, p, hs, x);
+        for (int q = q0; q < q1; q += kPtcPairs) {
+            __syncthreads();  // the last stage is read
+            Mat3<float> V;
+            int dl = 0, src = 0;  // direction whose link is in V
+#pragma unroll 1
+            for (int slot = st_slot; slot < kPtcPairs; slot += kPtcThreads / kPtcSites) {
+                const int d = (q + slot) / cin, cp = (q + slot) % cin;
+                cplx<float> t[12];
+                if (hs < g.Vh && q + slot < q1) {
+                    const float4* ac = a + cp * chs;
+                    if (d == 0) {
+                        load_spinor<1>(ac + (size_t)p * 6 * g.Vh, g.Vh, hs, t);
+                    } else {
+                        if (d != dl) {
+                            vlink_for(g, L, d, p, hs, x, V, src);
+                            dl = d;
+                        }
+                        cplx<float> v[12];
+                        load_spinor<1>(ac + (size_t)(1 - p) * 6 * g.Vh, g.Vh, src, v);
+                        transport_v(V, d <= 4, v, t);
+                    }
+                } else {
 #pragma unroll
-            for (int c = 0; c < COUT; ++c) {
-                if (c >= ng) break;
+                    for (int k = 0; k < 12; ++k) t[k] = {0.f, 0.f};
+                }
 #pragma unroll
-                for (int sp = 0; sp < 4; ++sp) {
-                    const float4 w01 = w[c * 8 + sp * 2], w23 = w[c * 8 + sp * 2 + 1];
-                    cmac(acc[c][sp], cplx<float>{w01.x, w01.y}, t[0]);
-                    cmac(acc[c][sp], cplx<float>{w01.z, w01.w}, t[1]);
-                    cmac(acc[c][sp], cplx<float>{w23.x, w23.y}, t[2]);
-                    cmac(acc[c][sp], cplx<float>{w23.z, w23.w}, t[3]);
+                for (int k = 0; k < 12; ++k) S.t[4 * slot + k / 3][k % 3][st_site] = make_float2(t[k].re, t[k].im);
+            }
+            const int np = min(kPtcPairs, q1 - q);
+            for (int e = tid; e < np * (kPlane / 4); e += kPtcThreads) {
+                const int slot = e / (kPlane / 4), r = e % (kPlane / 4), f = r / (4 * kPtcGroup), u = r % (4 * kPtcGroup);
+                const float4 v = QXD_LDG(reinterpret_cast<const float4*>(planes + ((size_t)blockIdx.z * 9 * cin + q + slot) * kPlane) + r);
+                *reinterpret_cast<float4*>(&S.w[f][4 * slot][0] + 4 * u) = v;
+            }
+            __syncthreads();
+#pragma unroll 2
+            for (int kk = 0; kk < 4 * kPtcPairs / KG; ++kk) {
+                const int k = kg * (4 * kPtcPairs / KG) + kk;
+                if (k >= 4 * np) break;
+                float2 w[3][R / 2];
+#pragma unroll
+                for (int f = 0; f < 3; ++f)
+#pragma unroll
+                    for (int r = 0; r < R / 4; ++r) {
+                        const float4 v = *reinterpret_cast<const float4*>(&S.w[f][k][R * cg + 4 * r]);
+                        w[f][2 * r] = make_float2(v.x, v.y);
+                        w[f][2 * r + 1] = make_float2(v.z, v.w);
+                    }
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const float2 t = S.t[k][i][site];
+                    const float2 tr = make_float2(t.x, t.x), ti = make_float2(t.y, t.y);
+#pragma unroll
+                    for (int r = 0; r < R / 2; ++r) {
+                        re[r][i] = fma2(w[2][r], ti, fma2(w[0][r], tr, re[r][i]));
+                        im[r][i] = fma2(w[1][r], tr, fma2(w[0][r], ti, im[r][i]));
+                    }
                 }
             }
         }
-    }
-    // complex (spin sp, colour I) is component (q & 1) of chunk q >> 1, q = 3 sp + I
+        if constexpr (KG > 1) {  // add the groups' sums, group 1 first
+            float2* red = &S.t[0][0][0];
+            constexpr int NV = 3 * R;  // float2 values of a thread
+            __syncthreads();
+            if (kg > 0) {
+                float2* o = red + (size_t)(((kg - 1) * CG + cg) * 2 + sg) * NV * 32 + lane;
 #pragma unroll
-    for (int c = 0; c < COUT; ++c) {
-        if (c >= ng) break;
-        float2* o = reinterpret_cast<float2*>(out + (c0 + c) * chs + (size_t)p * 6 * g.Vh);
+                for (int r = 0; r < R / 2; ++r)
 #pragma unroll
-        for (int sp = 0; sp < 4; ++sp) {
-            const int q = 3 * sp + I;
-            o[2 * ((size_t)(q >> 1) * g.Vh + h) + (q & 1)] = make_float2(acc[c][sp].re, acc[c][sp].im);
+                    for (int i = 0; i < 3; ++i) {
+                        o[(2 * (3 * r + i)) * 32] = re[r][i];
+                        o[(2 * (3 * r + i) + 1) * 32] = im[r][i];
+                    }
+            }
+            __syncthreads();
+            if (kg == 0) {
+                for (int k = 1; k < KG; ++k) {
+                    const float2* o = red + (size_t)(((k - 1) * CG + cg) * 2 + sg) * NV * 32 + lane;
+#pragma unroll
+                    for (int r = 0; r < R / 2; ++r)
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) {
+                            const float2 u = o[(2 * (3 * r + i)) * 32], v = o[(2 * (3 * r + i) + 1) * 32];
+                            re[r][i] = make_float2(re[r][i].x + u.x, re[r][i].y + u.y);
+                            im[r][i] = make_float2(im[r][i].x + v.x, im[r][i].y + v.y);
+                        }
+                }
+            }
         }
-    }
-}
-
-template <int COUT>
-__global__ void __launch_bounds__(kPtcFwdThreads) k_ptc_fwd(Geo g, PtcLinks L, const float4* __restrict__ a, int cin,
-                                                           int cout, const float2* __restrict__ W,
-                                                           float4* __restrict__ out) {
-    extern __shared__ float4 wsh4[];
-    float2* wsh = reinterpret_cast<float2*>(wsh4);
-    const int c0 = blockIdx.z * kPtcGroup;
-    const int ng = min(kPtcGroup, cout - c0);
-    // W[c][c'][d][s][s'] (global) -> wsh[d][c'][c - c0][s][s'] (zero for c >= ng)
-    const int nw = 9 * cin * COUT * 16;
-    for (int i = threadIdx.x; i < nw; i += blockDim.x) {
-        const int e = i % 16, c = (i / 16) % COUT, cp = (i / (16 * COUT)) % cin, d = i / (16 * COUT * cin);
-        wsh[i] = c < ng ? W[((size_t)((c0 + c) * cin + cp) * 9 + d) * 16 + e] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    const int colour = threadIdx.x / kPtcSites;
-    const int lane_site = threadIdx.x % kPtcSites;
-    const int tiles = (g.Vh + kPtcSites - 1) / kPtcSites;
-    for (int t = blockIdx.x; t < 2 * tiles; t += gridDim.x) {
-        const int p = t / tiles;
-        const int h = (t % tiles) * kPtcSites + lane_site;
-        if (h >= g.Vh) continue;
-        if (colour == 0) ptc_fwd_site<0, COUT>(g, L, a, cin, ng, wsh, out, c0, p, h);
-        else if (colour == 1) ptc_fwd_site<1, COUT>(g, L, a, cin, ng, wsh, out, c0, p, h);
-        else ptc_fwd_site<2, COUT>(g, L, a, cin, ng, wsh, out, c0, p, h);
-    }
-}
-
-// W'[c'][c][d'] = W[c][c'][opposite(d')]^+ (the adjoint layer as a forward layer)
-__global__ void k_ptc_adjoint_weights(const float2* __restrict__ W, int cin, int cout, float2* __restrict__ Wa) {
-    const int n = cout * cin * 9;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-        const int d = q % 9, cp = (q / 9) % cin, c = q / (9 * cin);
-        const int dop = d == 0 ? 0 : (d <= 4 ? d + 4 : d - 4);
-        const float2* src = W + ((size_t)(c * cin + cp) * 9 + d) * 16;
-        float2* dst = Wa + ((size_t)(cp * cout + c) * 9 + dop) * 16;
-        for (int s = 0; s < 4; ++s)
-            for (int t = 0; t < 4; ++t) dst[4 * t + s] = make_float2(src[4 * s + t].x, -src[4 * s + t].y);
+        if (kg == 0 && h0 + site < g.Vh) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                if (NC * cg + c >= ng) break;
+                cplx<float> v[12];
+#pragma unroll
+                for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        const float2 a2 = re[2 * c + sp / 2][i], b2 = im[2 * c + sp / 2][i];
+                        v[3 * sp + i] = (sp & 1) ? cplx<float>{a2.y, b2.y} : cplx<float>{a2.x, b2.x};
+                    }
+                store_spinor<1>(out + (c0 + NC * cg + c) * chs + (size_t)p * 6 * g.Vh, g.Vh, h0 + site, v);
+            }
+        }
     }
 }
 
 // ---- weight gradient ----------------------------------------------------------------
-// G[c][c'][d][s][s'] = sum_{x,i} delta_c(x)[s][i] conj((T_d a_{c'})(x)[s'][i]): for each d
-// the product of the (c,s) x (x,i) matrix of delta with the (x,i) x (c',s') matrix of
-// conjugated transports, summed over K = 3V rows in tiles of 3 kPtcSites rows.  A block
-// owns one chunk (blockIdx.z) of at most 32 (c,s) x 32 (c',s') entries for all nine d;
-// each of its 256 threads a 2 x 2 sub-block of the chunk for every d (36 complex
-// accumulators).  Per tile the delta rows are staged once and the transports once per
-// d, both in shared memory; T_d a_{c'} is formed once per site, colour, d and c'.
-// Sums run in FP32 within a block; the blocks' partials are added in FP64 in a fixed
-// order by k_ptc_wgrad_final.
+// G[c][c'][d][s][s'] = sum_{x,i} delta_c(x)[s][i] conj((T_d a_{c'})(x)[s'][i]): the product of
+// the (c, s) x (x, i) matrix of delta with the (x, i) x (d, c', s') matrix of conjugated
+// transports, summed over the 3V columns (x, i).  A block owns one chunk (blockIdx.z) of at
+// most 8 output and 8 input channels, all nine d, and every gridDim.x-th tile of sites.  The
+// transports of a tile (all d) and its delta are staged in shared memory; then a lane owns
+// two neighbouring (c', s') (one packed FP32 instruction) and all nine d for two spins of one
+// output channel, a warp all (c', s') of its channel: 36 complex sums per thread.  With CIP < 8 input or fewer
+// than 8 output channels the spare lanes and warps take other columns; their sums are added
+// at the end in a fixed order.  Sums run in FP32 within a block; the blocks' partials are
+// added in FP64 in a fixed order by k_ptc_wgrad_final.
+//
+// Bound by the FP32 pipe (194 us for 8 x 8 channels on 16^4).  With 2 x 2 sums per thread
+// and one d staged at a time the kernel was bound by shared-memory loads: 674 us whatever
+// the channel counts, and 94 us for the final sum in one thread per entry; here 417 us
+// for 8 x 8, 70 us for 1 -> 8 and 97 us for 8 -> 1 channels, the final sum 26 us.
 constexpr int kWgThreads = 256;
-constexpr int kWgRows = 3 * kPtcSites;
-constexpr size_t kWgSmem = 2ull * kWgRows * 32 * sizeof(float2);  // delta and transport tiles
+constexpr int kWgReal = 36;  // float2 sums of a thread: 9 d x 2 rows x (re, im), each for two (c', s')
 
-template <int I>
-__device__ void wgrad_stage(const Geo& g, const PtcLinks& L, const float4* __restrict__ delta,
-                            const float4* __restrict__ a, int d, int p, int h, bool live, int r_c0, int nr_c,
-                            int c_c0, int nc_c, float2 (*dsh)[32], float2 (*tsh)[32], int row) {
-    const size_t chs = (size_t)12 * g.Vh;
-    int x[4];
-    if (live) site_coords(g, p, h, x);
-    if (d < 0) {
-        // delta_c(x)[s][I] for the chunk's output channels
-        for (int c = 0; c < 8; ++c) {
-            cplx<float> t[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-            if (live && c < nr_c) {
-                PtcLink none;
-                transport_row<I>(g, 0, p, h, none, delta + (r_c0 + c) * chs, t);
-            }
-            for (int sp = 0; sp < 4; ++sp) dsh[row][c * 4 + sp] = make_float2(t[sp].re, t[sp].im);
-        }
-        return;
-    }
-    PtcLink lk;
-    if (live && d > 0) link_for(g, L, d, p, h, x, lk);
-    for (int c = 0; c < 8; ++c) {
-        cplx<float> t[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-        if (live && c < nc_c) transport_row<I>(g, d, p, h, lk, a + (c_c0 + c) * chs, t);
-        for (int sp = 0; sp < 4; ++sp) tsh[row][c * 4 + sp] = make_float2(t[sp].re, t[sp].im);
-    }
-}
+template <int CIP>
+struct WgShape {
+    static constexpr int SITES = CIP == 8 ? 8 : 16;
+    static constexpr int COLS = 3 * SITES;
+    static constexpr int K = 4 * CIP;            // (c', s') lanes of a column
+    static constexpr int CS = 2 * 9 * K + 4;     // floats per column: Re, Im planes (padded against bank conflicts)
+    static constexpr int NSUB = 8 / CIP;         // columns of a warp's lanes
+    static constexpr size_t T_BYTES = (size_t)COLS * CS * sizeof(float);
+    static constexpr size_t D_BYTES = 3ull * COLS * 32 * sizeof(float);  // Re, Im, -Re of delta
+    static constexpr size_t RED = 4ull * kWgReal * 32 * sizeof(float2);  // sums of half the warps
+    static constexpr size_t SMEM = T_BYTES + D_BYTES > RED ? T_BYTES + D_BYTES : RED;
+};
 
-__global__ void __launch_bounds__(kWgThreads) k_ptc_wgrad(Geo g, PtcLinks L, const float4* __restrict__ delta,
-                                                         const float4* __restrict__ a, int cin, int cout,
-                                                         float2* __restrict__ partials) {
+template <int CIP>
+__global__ void __launch_bounds__(kWgThreads, 2)
+    k_ptc_wgrad(Geo g, PtcLinks L, const float4* __restrict__ delta, const float4* __restrict__ a, int cin, int cout,
+                int rg, float2* __restrict__ partials, bool delta_even, bool a_even) {
+    using S = WgShape<CIP>;
     extern __shared__ float4 wg_sh[];
-    float2 (*dsh)[32] = reinterpret_cast<float2 (*)[32]>(wg_sh);
-    float2 (*tsh)[32] = dsh + kWgRows;
+    float* tsh = reinterpret_cast<float*>(wg_sh);
+    float* dsh = reinterpret_cast<float*>(reinterpret_cast<char*>(wg_sh) + S::T_BYTES);  // [3][COLS][32]
     const int nzc = (cin + 7) / 8;
     const int zr = blockIdx.z / nzc, zc = blockIdx.z % nzc;
     const int r_c0 = 8 * zr, nr_c = min(8, cout - r_c0);  // output channels of the chunk
     const int c_c0 = 8 * zc, nc_c = min(8, cin - c_c0);   // input channels of the chunk
-    const int tid = threadIdx.x;
-    const int r0 = 2 * (tid / 16), q0 = 2 * (tid % 16);  // this thread's 2 x 2 sub-block
-    cplx<float> acc[9][2][2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // rg warps (1, 2, 4 or 8) cover the output channels, the 8 / rg groups of them the columns
+    const int c = warp % rg, cs = warp / rg;
+    const int k = 2 * (lane % (S::K / 2)), rh = (lane % S::K) / (S::K / 2), sub = lane / S::K;
+    const int step = (8 / rg) * S::NSUB;
+    const size_t chs = (size_t)12 * g.Vh;
+    float2 re[9][2], im[9][2];
 #pragma unroll
     for (int d = 0; d < 9; ++d)
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) acc[d][i][j] = {0.f, 0.f};
-    const int colour = tid / kPtcSites;  // staging threads: tid < kWgRows
-    const int lane_site = tid % kPtcSites;
-    const int tiles = (g.Vh + kPtcSites - 1) / kPtcSites;
-    for (int t = blockIdx.x; t < 2 * tiles; t += gridDim.x) {
+        for (int r = 0; r < 2; ++r) re[d][r] = im[d][r] = make_float2(0.f, 0.f);
+    const int tiles = (g.Vh + S::SITES - 1) / S::SITES;
+    for (int t = blockIdx.x; t < (delta_even ? tiles : 2 * tiles); t += gridDim.x) {
         const int p = t / tiles;
-        const int h = (t % tiles) * kPtcSites + lane_site;
-        const bool live = h < g.Vh;
-        __syncthreads();  // the previous tile's rows are no longer read
-        if (tid < kWgRows) {
-            if (colour == 0) wgrad_stage<0>(g, L, delta, a, -1, p, h, live, r_c0, nr_c, c_c0, nc_c, dsh, tsh, tid);
-            else if (colour == 1) wgrad_stage<1>(g, L, delta, a, -1, p, h, live, r_c0, nr_c, c_c0, nc_c, dsh, tsh, tid);
-            else wgrad_stage<2>(g, L, delta, a, -1, p, h, live, r_c0, nr_c, c_c0, nc_c, dsh, tsh, tid);
-        }
+        const int h0 = (t % tiles) * S::SITES;
+        const int d0 = a_even && p == 1 ? 1 : 0, d1 = a_even && p == 0 ? 1 : 9;
+        __syncthreads();  // the last tile is read
+        for (int e = tid; e < S::SITES * 8; e += kWgThreads) {
+            const int site = e % S::SITES, ch = e / S::SITES;
+            cplx<float> v[12];
+            if (ch < nr_c && h0 + site < g.Vh)
+                load_spinor<1>(delta + (r_c0 + ch) * chs + (size_t)p * 6 * g.Vh, g.Vh, h0 + site, v);
+            else
 #pragma unroll
-        for (int d = 0; d < 9; ++d) {
-            __syncthreads();
-            if (tid < kWgRows) {
-                if (colour == 0) wgrad_stage<0>(g, L, delta, a, d, p, h, live, r_c0, nr_c, c_c0, nc_c, dsh, tsh, tid);
-                else if (colour == 1) wgrad_stage<1>(g, L, delta, a, d, p, h, live, r_c0, nr_c, c_c0, nc_c, dsh, tsh, tid);
-                else wgrad_stage<2>(g, L, delta, a, d, p, h, live, r_c0, nr_c, c_c0, nc_c, dsh, tsh, tid);
+                for (int q = 0; q < 12; ++q) v[q] = {0.f, 0.f};
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                float* o = dsh + (3 * site + i) * 32 + 4 * ch;
+                *reinterpret_cast<float4*>(o) = make_float4(v[i].re, v[3 + i].re, v[6 + i].re, v[9 + i].re);
+                *reinterpret_cast<float4*>(o + S::COLS * 32) =
+                    make_float4(v[i].im, v[3 + i].im, v[6 + i].im, v[9 + i].im);
+                *reinterpret_cast<float4*>(o + 2 * S::COLS * 32) =
+                    make_float4(-v[i].re, -v[3 + i].re, -v[6 + i].re, -v[9 + i].re);
             }
-            __syncthreads();
-#pragma unroll 4
-            for (int k = 0; k < kWgRows; ++k) {
-                const float4 dv = *reinterpret_cast<const float4*>(&dsh[k][r0]);
-                const float4 tv = *reinterpret_cast<const float4*>(&tsh[k][q0]);
-                const cplx<float> dd[2] = {{dv.x, dv.y}, {dv.z, dv.w}};
-                const cplx<float> tt[2] = {{tv.x, tv.y}, {tv.z, tv.w}};
+        }
+#pragma unroll 1
+        for (int e = tid + d0 * S::SITES * CIP; e < d1 * S::SITES * CIP; e += kWgThreads) {
+            const int site = e % S::SITES, cp = (e / S::SITES) % CIP, d = e / (S::SITES * CIP);
+            const int h = h0 + site;
+            cplx<float> v[12];
+            if (cp < nc_c && h < g.Vh) {
+                const float4* ac = a + (c_c0 + cp) * chs;
+                if (d == 0) {
+                    load_spinor<1>(ac + (size_t)p * 6 * g.Vh, g.Vh, h, v);
+                } else {
+                    int x[4], src;
+                    site_coords(g, p, h, x);
+                    Mat3<float> V;
+                    vlink_for(g, L, d, p, h, x, V, src);
+                    cplx<float> w[12];
+                    load_spinor<1>(ac + (size_t)(1 - p) * 6 * g.Vh, g.Vh, src, w);
+                    transport_v(V, d <= 4, w, v);
+                }
+            } else {
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
+                for (int q = 0; q < 12; ++q) v[q] = {0.f, 0.f};
+            }
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) cmac_conj(acc[d][i][j], tt[j], dd[i]);
+            for (int i = 0; i < 3; ++i) {
+                float* o = tsh + (size_t)(3 * site + i) * S::CS + d * S::K + 4 * cp;
+                *reinterpret_cast<float4*>(o) = make_float4(v[i].re, v[3 + i].re, v[6 + i].re, v[9 + i].re);
+                *reinterpret_cast<float4*>(o + 9 * S::K) = make_float4(v[i].im, v[3 + i].im, v[6 + i].im, v[9 + i].im);
+            }
+        }
+        __syncthreads();
+        for (int col = cs * S::NSUB + sub; col < S::COLS; col += step) {
+            const float* dp = dsh + col * 32 + 4 * c + 2 * rh;
+            const float2 fr = *reinterpret_cast<const float2*>(dp);
+            const float2 fi = *reinterpret_cast<const float2*>(dp + S::COLS * 32);
+            const float2 fn = *reinterpret_cast<const float2*>(dp + 2 * S::COLS * 32);
+            const float2 dr[2] = {{fr.x, fr.x}, {fr.y, fr.y}}, di[2] = {{fi.x, fi.x}, {fi.y, fi.y}},
+                         dn[2] = {{fn.x, fn.x}, {fn.y, fn.y}};
+            const float* tp = tsh + (size_t)col * S::CS + k;
+#pragma unroll
+            for (int d = 0; d < 9; ++d) {
+                if (d < d0 || d >= d1) continue;
+                const float2 tr = *reinterpret_cast<const float2*>(tp + d * S::K);
+                const float2 ti = *reinterpret_cast<const float2*>(tp + (9 + d) * S::K);
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {  // delta conj(T)
+                    re[d][r] = fma2(di[r], ti, fma2(dr[r], tr, re[d][r]));
+                    im[d][r] = fma2(dn[r], ti, fma2(di[r], tr, im[d][r]));
+                }
             }
         }
     }
+    // columns of the same warp, then of the other warps of the channel (group 1 first)
+#pragma unroll
+    for (int o = S::K; o < 32; o <<= 1)
+#pragma unroll
+        for (int d = 0; d < 9; ++d)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                re[d][r].x += __shfl_xor_sync(0xffffffffu, re[d][r].x, o);
+                re[d][r].y += __shfl_xor_sync(0xffffffffu, re[d][r].y, o);
+                im[d][r].x += __shfl_xor_sync(0xffffffffu, im[d][r].x, o);
+                im[d][r].y += __shfl_xor_sync(0xffffffffu, im[d][r].y, o);
+            }
+    float2* red = reinterpret_cast<float2*>(tsh);
+    for (int s = 1; s < 8 / rg; ++s) {  // group s hands its sums to group 0
+        __syncthreads();
+        if (cs == s) {
+            float2* o = red + (size_t)c * kWgReal * 32 + lane;
+#pragma unroll
+            for (int d = 0; d < 9; ++d)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    o[(4 * d + 2 * r) * 32] = re[d][r];
+                    o[(4 * d + 2 * r + 1) * 32] = im[d][r];
+                }
+        }
+        __syncthreads();
+        if (cs == 0) {
+            const float2* o = red + (size_t)c * kWgReal * 32 + lane;
+#pragma unroll
+            for (int d = 0; d < 9; ++d)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float2 u = o[(4 * d + 2 * r) * 32], v = o[(4 * d + 2 * r + 1) * 32];
+                    re[d][r] = make_float2(re[d][r].x + u.x, re[d][r].y + u.y);
+                    im[d][r] = make_float2(im[d][r].x + v.x, im[d][r].y + v.y);
+                }
+        }
+    }
+    if (cs != 0 || sub != 0) return;
     float2* out = partials + ((size_t)blockIdx.z * gridDim.x + blockIdx.x) * 9 * 1024;
 #pragma unroll
     for (int d = 0; d < 9; ++d)
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-                out[d * 1024 + (r0 + i) * 32 + (q0 + j)] = make_float2(acc[d][i][j].re, acc[d][i][j].im);
+        for (int r = 0; r < 2; ++r) {
+            *reinterpret_cast<float4*>(out + d * 1024 + (4 * c + 2 * rh + r) * 32 + k) =
+                make_float4(re[d][r].x, im[d][r].x, re[d][r].y, im[d][r].y);
+        }
 }
 
-// G (+)= sum over the blocks' partials in FP64, blocks in a fixed order
-__global__ void k_ptc_wgrad_final(const float2* __restrict__ partials, int nblk, int cin, int cout,
-                                  float2* __restrict__ G, int accumulate) {
-    const int nzc = (cin + 7) / 8, nz = ((cout + 7) / 8) * nzc;
-    const int n = nz * 9 * 1024;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        const int e = t % 1024, d = (t / 1024) % 9, z = t / (9 * 1024);
-        const int r = e / 32, q = e % 32;
-        const int c = 8 * (z / nzc) + r / 4, cp = 8 * (z % nzc) + q / 4;
-        if (c >= cout || cp >= cin) continue;
-        double re = 0.0, im = 0.0;
-        for (int b = 0; b < nblk; ++b) {
-            const float2 v = partials[((size_t)z * nblk + b) * 9 * 1024 + d * 1024 + e];
+// G (+)= sum over the blocks' partials in FP64: 32 entries per block, eight threads per entry
+// over every eighth partial, their sums added in a fixed order
+__global__ void __launch_bounds__(256) k_ptc_wgrad_final(const float2* __restrict__ partials, int nblk, int cin,
+                                                         int cout, float2* __restrict__ G, int accumulate) {
+    __shared__ double2 sh[8][32];
+    const int nzc = (cin + 7) / 8;
+    const int q = threadIdx.x & 31, part = threadIdx.x >> 5;
+    const int r = blockIdx.x % 32, d = (blockIdx.x / 32) % 9, z = blockIdx.x / (32 * 9);
+    const int c = 8 * (z / nzc) + r / 4, cp = 8 * (z % nzc) + q / 4;
+    const bool live = c < cout && cp < cin;
+    double re = 0.0, im = 0.0;
+    if (live)
+        for (int b = part; b < nblk; b += 8) {
+            const float2 v = partials[((size_t)z * nblk + b) * 9 * 1024 + d * 1024 + r * 32 + q];
             re += v.x;
             im += v.y;
         }
-        const size_t o = ((size_t)(c * cin + cp) * 9 + d) * 16 + (r % 4) * 4 + (q % 4);
-        const float2 g0 = accumulate ? G[o] : make_float2(0.f, 0.f);
-        G[o] = make_float2(g0.x + (float)re, g0.y + (float)im);
+    sh[part][q] = make_double2(re, im);
+    __syncthreads();
+    if (part != 0 || !live) return;
+    for (int k = 1; k < 8; ++k) {
+        re += sh[k][q].x;
+        im += sh[k][q].y;
     }
+    const size_t o = ((size_t)(c * cin + cp) * 9 + d) * 16 + (r % 4) * 4 + (q % 4);
+    const float2 g0 = accumulate ? G[o] : make_float2(0.f, 0.f);
+    G[o] = make_float2(g0.x + (float)re, g0.y + (float)im);
 }
 
 // ---- forward layer on the tensor cores (tcgen05) ------------------------------------
@@ -649,21 +850,20 @@ static PtcLinks links_of(qxd_ctx* ctx, int fl) { return PtcLinks{ctx->U32, ctx->
 
 static size_t chan_bytes(const qxd_ctx* ctx) { return (size_t)ctx->g.Vh * 2 * 96; }
 
-// one forward layer: COUT = output channels per block (the smallest of 1, 2, 4, 8 that
-// holds min(cout, 8)), grid.z = groups of 8 output channels, a persistent grid of
-// resident blocks over the tiles of both parities
-template <int COUT>
-static int launch_fwd(qxd_ctx* ctx, int fl, const float4* a, int cin, const float2* W, float4* out, int cout,
-                      cudaStream_t st) {
+// one forward layer: grid.z = groups of 8 output channels, a persistent grid of resident
+// blocks over the tiles of the wanted parities
+template <int NC, int CG, int KG>
+static int launch_fwd(qxd_ctx* ctx, int fl, const float4* a, int cin, const float* W, float4* out, int cout,
+                      PtcParity par, cudaStream_t st) {
     const Geo& g = ctx->g;
-    const size_t smem = 9ull * cin * COUT * 16 * sizeof(float2);
-    QXD_CUDA(ctx, cudaFuncSetAttribute(k_ptc_fwd<COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int smem = (int)sizeof(PtcFwdShared);
+    QXD_CUDA(ctx, cudaFuncSetAttribute(k_ptc_fwd<NC, CG, KG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     int per_sm = 0;
-    QXD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ptc_fwd<COUT>, kPtcFwdThreads, smem));
+    QXD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ptc_fwd<NC, CG, KG>, kPtcThreads, smem));
     const int groups = (cout + kPtcGroup - 1) / kPtcGroup;
-    const int tiles = 2 * ((g.Vh + kPtcSites - 1) / kPtcSites);
+    const int tiles = (par.out_even ? 1 : 2) * ((g.Vh + kPtcSites - 1) / kPtcSites);
     const int nx = std::max(1, std::min(tiles, std::max(1, per_sm) * ctx->nsm / groups));
-    k_ptc_fwd<COUT><<<dim3(nx, 1, groups), kPtcFwdThreads, smem, st>>>(g, links_of(ctx, fl), a, cin, cout, W, out);
+    k_ptc_fwd<NC, CG, KG><<<dim3(nx, 1, groups), kPtcThreads, smem, st>>>(g, links_of(ctx, fl), a, cin, cout, W, out, par);
     QXD_CUDA(ctx, cudaGetLastError());
     return QXD_OK;
 }
@@ -673,14 +873,24 @@ static double layer_bytes(const qxd_ctx* ctx, int cin, int cout) {
     return (double)chan_bytes(ctx) * (cin + cout) + (double)ctx->g.V * 4 * 56;
 }
 
-static int launch_layer(qxd_ctx* ctx, int fl, const float4* a, int cin, const float2* W, float4* out, int cout,
-                        cudaStream_t st) {
+// floats of a layer's weight planes, and their preparation (adjoint: of the adjoint layer)
+static size_t plane_floats(int cin, int cout) {
+    return (size_t)((cout + kPtcGroup - 1) / kPtcGroup) * 9 * cin * kPlane;
+}
+static int launch_planes(qxd_ctx* ctx, const float2* W, int cin, int cout, bool adjoint, float* P, cudaStream_t st) {
+    const long long n = (long long)plane_floats(cin, cout) / 3;
+    k_ptc_planes<<<nblocks(n, 256), 256, 0, st>>>(W, cin, cout, adjoint ? 1 : 0, P);
+    QXD_CUDA(ctx, cudaGetLastError());
+    return QXD_OK;
+}
+
+static int launch_layer(qxd_ctx* ctx, int fl, const float4* a, int cin, const float* W, float4* out, int cout,
+                        PtcParity par, cudaStream_t st) {
     ProfScope prof(ctx, "ptc_layer", layer_bytes(ctx, cin, cout), st);
-    const int cg = std::min(cout, kPtcGroup);
-    if (cg <= 1) return launch_fwd<1>(ctx, fl, a, cin, W, out, cout, st);
-    if (cg <= 2) return launch_fwd<2>(ctx, fl, a, cin, W, out, cout, st);
-    if (cg <= 4) return launch_fwd<4>(ctx, fl, a, cin, W, out, cout, st);
-    return launch_fwd<8>(ctx, fl, a, cin, W, out, cout, st);
+    if (cout == 1) return launch_fwd<1, 1, 4>(ctx, fl, a, cin, W, out, cout, par, st);
+    if (cout == 2) return launch_fwd<2, 1, 4>(ctx, fl, a, cin, W, out, cout, par, st);
+    if (cout <= 4) return launch_fwd<2, 2, 2>(ctx, fl, a, cin, W, out, cout, par, st);
+    return launch_fwd<2, 4, 1>(ctx, fl, a, cin, W, out, cout, par, st);
 }
 
 // one forward layer on the tensor cores (bfloat16 operands, FP32 accumulation): input
@@ -707,7 +917,6 @@ static int launch_fwd_tc(qxd_ctx* ctx, int fl, const float4* a, int cin, const f
 
 static int launch_layer_tc(qxd_ctx* ctx, int fl, const float4* a, int cin, const float2* W, float4* out, int cout,
                            cudaStream_t st) {
-    if (cin > 8 || cout > 8) return launch_layer(ctx, fl, a, cin, W, out, cout, st);
     ProfScope prof(ctx, "ptc_layer_tc", layer_bytes(ctx, cin, cout), st);
     if (cin <= 2 && cout <= 2) return launch_fwd_tc<2, 2>(ctx, fl, a, cin, W, out, cout, st);
     if (cin <= 2) return launch_fwd_tc<2, 8>(ctx, fl, a, cin, W, out, cout, st);
@@ -716,40 +925,76 @@ static int launch_layer_tc(qxd_ctx* ctx, int fl, const float4* a, int cin, const
 }
 
 // weight gradient of one layer into G (accumulated): grid (blocks, 1, chunks)
-static int wgrad_blocks(const qxd_ctx* ctx) {
-    const int tiles = 2 * ((ctx->g.Vh + kPtcSites - 1) / kPtcSites);
-    return std::max(1, std::min(tiles, 2 * ctx->nsm));
-}
+static int wgrad_blocks(const qxd_ctx* ctx) { return std::max(1, std::min(2 * ((ctx->g.Vh + 7) / 8), 2 * ctx->nsm)); }
 
 static size_t wgrad_partial_bytes(const qxd_ctx* ctx, int cin, int cout) {
     const size_t nz = (size_t)((cout + 7) / 8) * ((cin + 7) / 8);
     return nz * wgrad_blocks(ctx) * 9 * 1024 * sizeof(float2);
 }
 
-static int launch_wgrad(qxd_ctx* ctx, int fl, const float4* delta, const float4* a, int cin, int cout, float2* part,
-                        float2* G, cudaStream_t st) {
-    const Geo& g = ctx->g;
-    ProfScope prof(ctx, "ptc_wgrad", layer_bytes(ctx, cin, cout), st);
-    QXD_CUDA(ctx, cudaFuncSetAttribute(k_ptc_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem));
-    const int nblk = wgrad_blocks(ctx);
+template <int CIP>
+static int launch_wgrad_k(qxd_ctx* ctx, int fl, const float4* delta, const float4* a, int cin, int cout, float2* part,
+                          bool delta_even, bool a_even, cudaStream_t st) {
+    const int smem = (int)WgShape<CIP>::SMEM;
+    QXD_CUDA(ctx, cudaFuncSetAttribute(k_ptc_wgrad<CIP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int nz = ((cout + 7) / 8) * ((cin + 7) / 8);
-    k_ptc_wgrad<<<dim3(nblk, 1, nz), kWgThreads, kWgSmem, st>>>(g, links_of(ctx, fl), delta, a, cin, cout, part);
-    QXD_CUDA(ctx, cudaGetLastError());
-    k_ptc_wgrad_final<<<nblocks((long long)nz * 9 * 1024, 256), 256, 0, st>>>(part, nblk, cin, cout, G, 1);
+    const int rg = cout > 4 ? 8 : cout > 2 ? 4 : cout;  // warps over the output channels
+    k_ptc_wgrad<CIP><<<dim3(wgrad_blocks(ctx), 1, nz), kWgThreads, smem, st>>>(ctx->g, links_of(ctx, fl), delta, a, cin,
+                                                                              cout, rg, part, delta_even, a_even);
     QXD_CUDA(ctx, cudaGetLastError());
     return QXD_OK;
 }
 
-// Forward pass: acts[0] = embedded input (1 channel); acts[l+1] = layer l (acts[l]).
-// prec QXD_FP32: CUDA-core FP32 layers; QXD_BF16: the channel mixing on the tensor cores
-static int ptc_forward(qxd_ctx* ctx, int fl, const float2* W, int nlayers, int nch, float4* const* acts,
-                       cudaStream_t st, int prec = QXD_FP32) {
+static int launch_wgrad(qxd_ctx* ctx, int fl, const float4* delta, const float4* a, int cin, int cout, float2* part,
+                        float2* G, bool delta_even, bool a_even, cudaStream_t st) {
+    ProfScope prof(ctx, "ptc_wgrad", layer_bytes(ctx, cin, cout), st);
+    if (cin == 1) QXD_TRY(launch_wgrad_k<1>(ctx, fl, delta, a, cin, cout, part, delta_even, a_even, st));
+    else if (cin == 2) QXD_TRY(launch_wgrad_k<2>(ctx, fl, delta, a, cin, cout, part, delta_even, a_even, st));
+    else if (cin <= 4) QXD_TRY(launch_wgrad_k<4>(ctx, fl, delta, a, cin, cout, part, delta_even, a_even, st));
+    else QXD_TRY(launch_wgrad_k<8>(ctx, fl, delta, a, cin, cout, part, delta_even, a_even, st));
+    const int nz = ((cout + 7) / 8) * ((cin + 7) / 8);
+    k_ptc_wgrad_final<<<nz * 9 * 32, 256, 0, st>>>(part, wgrad_blocks(ctx), cin, cout, G, 1);
+    QXD_CUDA(ctx, cudaGetLastError());
+    return QXD_OK;
+}
+
+// weight planes of all layers (adjoint: of the adjoints of layers 1 .. nlayers - 1) in
+// workspace `slot`; offsets by layer in off
+static int ptc_planes(qxd_ctx* ctx, const float2* W, int nlayers, int nch, bool adjoint, int slot, float** planes,
+                      std::vector<size_t>& off, cudaStream_t st) {
+    off.assign(nlayers + 1, 0);
+    for (int l = 0; l < nlayers; ++l) {
+        int ci, co;
+        layer_shape(l, nlayers, nch, &ci, &co);
+        off[l + 1] = off[l] + (adjoint ? plane_floats(co, ci) : plane_floats(ci, co));
+    }
+    void* P;
+    QXD_TRY(qxd_ws(ctx, slot, off[nlayers] * sizeof(float), &P));
+    *planes = static_cast<float*>(P);
     const float2* w = W;
     for (int l = 0; l < nlayers; ++l) {
         int ci, co;
         layer_shape(l, nlayers, nch, &ci, &co);
-        if (prec == QXD_BF16) QXD_TRY(launch_layer_tc(ctx, fl, acts[l], ci, w, acts[l + 1], co, st));
-        else QXD_TRY(launch_layer(ctx, fl, acts[l], ci, w, acts[l + 1], co, st));
+        if (!adjoint) QXD_TRY(launch_planes(ctx, w, ci, co, false, *planes + off[l], st));
+        else if (l > 0) QXD_TRY(launch_planes(ctx, w, co, ci, true, *planes + off[l], st));
+        w += layer_weights(ci, co);
+    }
+    return QXD_OK;
+}
+
+// Forward pass: acts[0] = embedded input (1 channel); acts[l+1] = layer l (acts[l]), of the
+// last layer the even sites.  planes: CUDA-core FP32 layers; else the channel mixing of
+// layers with at most 8 channels on the tensor cores with the weights W
+static int ptc_forward(qxd_ctx* ctx, int fl, const float2* W, const float* planes, const std::vector<size_t>& off,
+                       int nlayers, int nch, float4* const* acts, cudaStream_t st, bool tc) {
+    const float2* w = W;
+    for (int l = 0; l < nlayers; ++l) {
+        int ci, co;
+        layer_shape(l, nlayers, nch, &ci, &co);
+        if (tc && ci <= 8 && co <= 8) QXD_TRY(launch_layer_tc(ctx, fl, acts[l], ci, w, acts[l + 1], co, st));
+        else
+            QXD_TRY(launch_layer(ctx, fl, acts[l], ci, planes + off[l], acts[l + 1], co,
+                                 PtcParity{l == 0 && nlayers > 1, l == nlayers - 1}, st));
         w += layer_weights(ci, co);
     }
     return QXD_OK;
@@ -782,7 +1027,10 @@ int ptc_apply_internal(qxd_ctx* ctx, int fl, const float2* W, int nlayers, int n
     QXD_CUDA(ctx, cudaMemcpyAsync(acts[0], r_e, hb, cudaMemcpyDeviceToDevice, st));
     QXD_CUDA(ctx, cudaMemsetAsync(reinterpret_cast<char*>(acts[0]) + hb, 0, hb, st));
     if (prec == QXD_BF16) QXD_CUDA(ctx, cudaMemsetAsync(ctx->dev_flag, 0, sizeof(int), st));
-    QXD_TRY(ptc_forward(ctx, fl, W, nlayers, nch, acts.data(), st, prec));
+    float* planes = nullptr;
+    std::vector<size_t> off;
+    if (prec != QXD_BF16 || nch > 8) QXD_TRY(ptc_planes(ctx, W, nlayers, nch, false, WS_PTC + 16, &planes, off, st));
+    QXD_TRY(ptc_forward(ctx, fl, W, planes, off, nlayers, nch, acts.data(), st, prec == QXD_BF16));
     QXD_CUDA(ctx, cudaMemcpyAsync(z_e, acts[nlayers], hb, cudaMemcpyDeviceToDevice, st));
     return QXD_OK;
 }
@@ -797,10 +1045,9 @@ static int ptc_loss_grad_internal(qxd_ctx* ctx, int fl, const float2* W, int nla
     const size_t n = 12ull * g.Vh;
     std::vector<float4*> acts;
     QXD_TRY(ptc_buffers(ctx, nlayers, nch, WS_PTC, acts));
-    void *dA, *dB, *Wa, *part;
+    void *dA, *dB, *part;
     QXD_TRY(qxd_ws(ctx, WS_PTC + 10, chan_bytes(ctx) * nch, &dA));
     QXD_TRY(qxd_ws(ctx, WS_PTC + 11, chan_bytes(ctx) * nch, &dB));
-    QXD_TRY(qxd_ws(ctx, WS_PTC + 12, layer_weights(nch, nch) * sizeof(float2), &Wa));
     QXD_TRY(qxd_ws(ctx, WS_PTC + 13, wgrad_partial_bytes(ctx, nch, nch), &part));
     // offsets of each layer's weights
     std::vector<size_t> off(nlayers + 1, 0);
@@ -809,12 +1056,17 @@ static int ptc_loss_grad_internal(qxd_ctx* ctx, int fl, const float2* W, int nla
         layer_shape(l, nlayers, nch, &ci, &co);
         off[l + 1] = off[l] + layer_weights(ci, co);
     }
+    // the weights of all pairs, in the layers' order
+    float *planes, *adj = nullptr;
+    std::vector<size_t> poff, aoff;
+    QXD_TRY(ptc_planes(ctx, W, nlayers, nch, false, WS_PTC + 16, &planes, poff, st));
+    if (G) QXD_TRY(ptc_planes(ctx, W, nlayers, nch, true, WS_PTC + 17, &adj, aoff, st));
     double tot = 0.0;
     for (int k = 0; k < nb; ++k) {
         const int i = idx[k];
         QXD_CUDA(ctx, cudaMemcpyAsync(acts[0], r + (size_t)i * hb, hb, cudaMemcpyDeviceToDevice, st));
         QXD_CUDA(ctx, cudaMemsetAsync(reinterpret_cast<char*>(acts[0]) + hb, 0, hb, st));
-        QXD_TRY(ptc_forward(ctx, fl, W, nlayers, nch, acts.data(), st));
+        QXD_TRY(ptc_forward(ctx, fl, W, planes, poff, nlayers, nch, acts.data(), st, false));
         float4* delta = static_cast<float4*>(dA);
         if (kind == 1) {
             // residual norm: res = Dhat (M r)_e - r; delta = Dhat^+ res / |r|^2 on even sites
@@ -847,13 +1099,10 @@ static int ptc_loss_grad_internal(qxd_ctx* ctx, int fl, const float2* W, int nla
         for (int l = nlayers - 1; l >= 0; --l) {
             int ci, co;
             layer_shape(l, nlayers, nch, &ci, &co);
-            const int nq = co * ci * 9;
-            QXD_TRY(launch_wgrad(ctx, fl, dcur, acts[l], ci, co, static_cast<float2*>(part), G + off[l], st));
+            QXD_TRY(launch_wgrad(ctx, fl, dcur, acts[l], ci, co, static_cast<float2*>(part), G + off[l],
+                                 l == nlayers - 1, l == 0, st));
             if (l > 0) {
-                k_ptc_adjoint_weights<<<nblocks(nq, 128), 128, 0, st>>>(W + off[l], ci, co,
-                                                                        static_cast<float2*>(Wa));
-                QXD_CUDA(ctx, cudaGetLastError());
-                QXD_TRY(launch_layer(ctx, fl, dcur, co, static_cast<float2*>(Wa), dnext, ci, st));
+                QXD_TRY(launch_layer(ctx, fl, dcur, co, adj + aoff[l], dnext, ci, PtcParity{l == nlayers - 1, false}, st));
                 std::swap(dcur, dnext);
             }
         }
