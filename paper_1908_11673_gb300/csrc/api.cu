@@ -29,12 +29,19 @@ int qxd_fail(qxd_ctx* ctx, int code, const std::string& msg) {
 }
 
 // Device memory of `bytes` bytes; when there is none left, the field buffers that
-// qxd_set_links kept for flavours not set again since are given back first.
+// qxd_set_links kept for flavours not set again since and the SAP copies (the sweeps do
+// without) are given back first.
 bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes) {
     if (cudaMalloc(p, bytes) == cudaSuccess) return true;
     cudaGetLastError();
-    for (auto& F : ctx->fl)
+    for (auto& F : ctx->fl) {
         if (!F.set && !F.building) free_fields(F);
+        if (F.sap) {
+            cudaFree(F.sap);
+            F.sap = nullptr;
+            F.sap_off = true;
+        }
+    }
     if (cudaMalloc(p, bytes) == cudaSuccess) return true;
     cudaGetLastError();
     *p = nullptr;
@@ -184,6 +191,7 @@ static void reset_flavour(QxdFlavour& F) {
     cudaFree(F.Cdf[0]);
     cudaFree(F.Cdf[1]);
     cudaFree(F.Vdf);
+    cudaFree(F.sap);
     cudaFree(F.W);
     cudaFree(F.dfl_basis);
     cudaFree(F.dfl_A);
@@ -298,12 +306,15 @@ int qxd_set_clover(qxd_ctx* ctx, int fl, const qxd_flavour* f, void* stream) {
         }
     }
     F.f = *f;
-    // double-float copies and a deflation subspace belong to the operator they were built for
+    // double-float and SAP copies and a deflation subspace belong to the operator they were built for
     cudaFree(F.Vdf);
     cudaFree(F.Cdf[0]);
     cudaFree(F.Cdf[1]);
     F.Vdf = nullptr;
     F.Cdf[0] = F.Cdf[1] = nullptr;
+    cudaFree(F.sap);
+    F.sap = nullptr;
+    F.sap_off = false;
     dfl_free(F);
     const int rc = launch_set_flavour(ctx, fl, st);
     F.building = false;
