@@ -135,6 +135,7 @@ enum {
     WS_SAP = 272,
     WS_RAT = 288,
     WS_DFL = 300,
+    WS_CG = 314,
     WS_CLOVER = 318,
     WS_NSLOTS = 320
 };

@@ -155,6 +155,8 @@ int cgnr_inner(qxd_ctx* ctx, int fl, int P, const void* b, void* e, int max_iter
     QXD_TRY(qxd_ws(ctx, WS_SOLVER + 102, hb, &p));
     QXD_TRY(qxd_ws(ctx, WS_SOLVER + 103, hb, &w));
     QXD_TRY(qxd_ws(ctx, WS_SOLVER + 104, hb, &to));
+    if (P == QXD_FP32)
+        return cg_lockstep(ctx, fl, 1, true, nullptr, &rtol, b, e, CgFields{sv, z, p, w, to}, max_iter, iters, st);
     QXD_CUDA(ctx, cudaMemsetAsync(e, 0, hb, st));
     QXD_CUDA(ctx, cudaMemcpyAsync(sv, b, hb, cudaMemcpyDeviceToDevice, st));
     QXD_TRY(op_Dhat(ctx, fl, P, 1, sv, z, to, st));
@@ -524,51 +526,6 @@ int op_normal(qxd_ctx* ctx, int fl, int P, double sigma, const void* v, void* ou
     return QXD_OK;
 }
 
-// CG on (Dhat^+ Dhat + sigma) e = b in precision P; e overwritten; stops at
-// |b - (A + sigma) e| <= rtol |b| (recursive residual).
-static int cg_shifted(qxd_ctx* ctx, int fl, int P, double sigma, const void* b, void* e, int max_iter, double rtol,
-                      int* iters, cudaStream_t st) {
-    const size_t n = 12ull * ctx->g.Vh;
-    const size_t hb = half_bytes(ctx, P);
-    void *r, *p, *Ap, *te, *to;
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 115, hb, &r));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 116, hb, &p));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 117, hb, &Ap));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 118, hb, &te));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 119, hb, &to));
-    QXD_CUDA(ctx, cudaMemsetAsync(e, 0, hb, st));
-    QXD_CUDA(ctx, cudaMemcpyAsync(r, b, hb, cudaMemcpyDeviceToDevice, st));
-    QXD_CUDA(ctx, cudaMemcpyAsync(p, b, hb, cudaMemcpyDeviceToDevice, st));
-    QXD_TRY(blas_norm2(ctx, P, n, b, 0, st));
-    QXD_TRY(blas_fetch(ctx, 2, st));
-    const double bn = std::sqrt(ctx->red_host[0]);
-    double rr = ctx->red_host[0];
-    *iters = 0;
-    if (bn == 0.0) return QXD_OK;
-    const double mone = -1.0;
-    while (*iters < max_iter) {
-        QXD_TRY(op_normal(ctx, fl, P, sigma, p, Ap, te, to, st));
-        QXD_TRY(blas_dot(ctx, P, P, n, p, Ap, 0, st));
-        QXD_TRY(blas_fetch(ctx, 2, st));
-        const double pAp = ctx->red_host[0];
-        *iters += 1;
-        if (!(pAp > 0.0)) return qxd_fail(ctx, QXD_EBREAKDOWN, "shifted CG: <p, A p> <= 0");
-        const double alpha = rr / pAp;
-        QXD_TRY(blas_axpby(ctx, P, P, n, alpha, 0.0, p, 1.0, 0.0, e, st));
-        const double ca = -alpha, ci = 0.0;
-        const void* Xp[1] = {Ap};
-        QXD_TRY(blas_multi_axpy_norm(ctx, P, n, 1, &ca, &ci, Xp, r, 0, st));
-        QXD_TRY(blas_fetch(ctx, 2, st));
-        QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "shifted CG"));
-        const double rr_new = ctx->red_host[0];
-        if (std::sqrt(rr_new) <= rtol * bn) break;
-        QXD_TRY(blas_axpby(ctx, P, P, n, 1.0, 0.0, r, rr_new / rr, 0.0, p, st));
-        rr = rr_new;
-    }
-    (void)mone;
-    return QXD_OK;
-}
-
 // Multi-shift CG in precision P on (Dhat^+ Dhat + sigma_j) x_j = b (Jegerlehner's
 // recursion: one Krylov space built with the smallest shift, the others
 // following through the scalars zeta_j).  X: ns fields of precision P (output).
@@ -838,6 +795,8 @@ static int mscg_core_graph(qxd_ctx* ctx, int fl, int P, int ns, const double* si
     return rc;
 }
 
+constexpr size_t kRefineBytes = 2ull << 30;
+
 int solve_mscg(qxd_ctx* ctx, int fl, int ns, const double* sigma, const qxd_solver* s, const void* b64, char* X64,
                qxd_info* info, cudaStream_t st) {
     const size_t n = 12ull * ctx->g.Vh;
@@ -876,12 +835,10 @@ int solve_mscg(qxd_ctx* ctx, int fl, int ns, const double* sigma, const qxd_solv
             QXD_TRY(blas_axpby(ctx, P, 0, n, 1.0, 0.0, static_cast<char*>(XP) + j * hbP, 0.0, 0.0, X64 + j * hb64, st));
     }
     // FP64 residual of every shift; FP32 defect correction where it misses tol
-    void *r64, *te, *to, *eP, *rP;
+    void *r64, *te, *to;
     QXD_TRY(qxd_ws(ctx, WS_SOLVER + 104, hb64, &r64));
     QXD_TRY(qxd_ws(ctx, WS_SOLVER + 105, hb64, &te));
     QXD_TRY(qxd_ws(ctx, WS_SOLVER + 106, hb64, &to));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 120, half_bytes(ctx, QXD_FP32), &eP));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 121, half_bytes(ctx, QXD_FP32), &rP));
     // With an FP32 Krylov space the residuals b - (Q2 + s_j) x_j are taken on the FP64
     // data in double-float arithmetic (FP32 pipe); they land in FP32 directly for the
     // correction solve.  A plain FP64 run keeps FP64.
@@ -894,36 +851,65 @@ int solve_mscg(qxd_ctx* ctx, int fl, int ns, const double* sigma, const qxd_solv
         QXD_TRY(qxd_ws(ctx, WS_SOLVER + 39, hb64, &tdf));
         QXD_TRY(blas_split_df64(ctx, b64, bdf, n, st));
     }
+    // the corrections of a group of shifts run in lockstep (one operator application for all of
+    // them); groups of at most kRefineBytes per field block, so that the workspace stays small
+    // on large lattices
+    const size_t h32 = half_bytes(ctx, QXD_FP32);
+    const int group = (int)std::max<size_t>(1, std::min<size_t>(ns, kRefineBytes / h32));
+    CgFields work{};
+    void *rb, *eb;
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 121, h32 * group, &rb));
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 120, h32 * group, &eb));
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 115, h32 * group, &work.r));
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 116, h32 * group, &work.p));
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 117, h32 * group, &work.w));
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 118, h32 * group, &work.t));
     double worst = 0.0;
-    for (int j = 0; j < ns; ++j) {
-        char* xj = X64 + j * hb64;
-        for (int pass = 0; pass < 16; ++pass) {
-            if (df) {
-                QXD_TRY(blas_split_df64(ctx, xj, xdf, n, st));
-                QXD_TRY(op_Dhat(ctx, fl, QXD_DF64, 0, xdf, tdf, to, st));
-                QXD_TRY(op_Dhat(ctx, fl, QXD_DF64, 1, tdf, ydf, to, st));
-                QXD_TRY(blas_df_shift_residual(ctx, bdf, ydf, xdf, sigma[j], rP, 0, st));
-            } else {
-                QXD_TRY(op_normal(ctx, fl, 0, sigma[j], xj, r64, te, to, st));
-                QXD_TRY(blas_axpby(ctx, 0, 0, n, 1.0, 0.0, b64, -1.0, 0.0, r64, st));
-                QXD_TRY(blas_norm2(ctx, 0, n, r64, 0, st));
+    for (int j0 = 0; j0 < ns; j0 += group) {
+        std::vector<int> open;  // shifts of the group that miss the tolerance
+        for (int j = j0; j < std::min(ns, j0 + group); ++j) open.push_back(j);
+        for (int pass = 0; pass < 16 && !open.empty(); ++pass) {
+            std::vector<int> next;
+            std::vector<double> sig, rtol, rels;
+            for (int j : open) {
+                char* xj = X64 + j * hb64;
+                char* rP = static_cast<char*>(rb) + next.size() * h32;
+                if (df) {
+                    QXD_TRY(blas_split_df64(ctx, xj, xdf, n, st));
+                    QXD_TRY(op_Dhat(ctx, fl, QXD_DF64, 0, xdf, tdf, to, st));
+                    QXD_TRY(op_Dhat(ctx, fl, QXD_DF64, 1, tdf, ydf, to, st));
+                    QXD_TRY(blas_df_shift_residual(ctx, bdf, ydf, xdf, sigma[j], rP, 0, st));
+                } else {
+                    QXD_TRY(op_normal(ctx, fl, 0, sigma[j], xj, r64, te, to, st));
+                    QXD_TRY(blas_axpby(ctx, 0, 0, n, 1.0, 0.0, b64, -1.0, 0.0, r64, st));
+                    QXD_TRY(blas_norm2(ctx, 0, n, r64, 0, st));
+                }
+                QXD_TRY(blas_fetch(ctx, 2, st));
+                QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "MSCG residual"));
+                const double rel = std::sqrt(ctx->red_host[0]) / bn;
+                if (verbose()) std::fprintf(stderr, "[qxd mscg] shift %d pass %d relres %.3e\n", j, pass, rel);
+                if (rel <= s->tol || info->iters >= s->nmx) {
+                    worst = std::max(worst, rel);
+                    continue;
+                }
+                info->restarts += 1;
+                if (!df) QXD_TRY(blas_axpby(ctx, 0, 1, n, 1.0, 0.0, r64, 0.0, 0.0, rP, st));
+                next.push_back(j);
+                sig.push_back(sigma[j]);
+                rtol.push_back(std::max(1e-5, 0.5 * s->tol / rel));
+                rels.push_back(rel);
             }
-            QXD_TRY(blas_fetch(ctx, 2, st));
-            QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "MSCG residual"));
-            const double rel = std::sqrt(ctx->red_host[0]) / bn;
-            if (verbose()) std::fprintf(stderr, "[qxd mscg] shift %d pass %d relres %.3e\n", j, pass, rel);
-            if (rel <= s->tol || info->iters >= s->nmx) {
-                worst = std::max(worst, rel);
-                break;
+            open = next;
+            if (open.empty()) break;
+            std::vector<int> its(open.size(), 0);
+            QXD_TRY(cg_lockstep(ctx, fl, (int)open.size(), false, sig.data(), rtol.data(), rb, eb, work,
+                                s->nmx - info->iters, its.data(), st));
+            for (size_t i = 0; i < open.size(); ++i) {
+                info->iters += its[i];
+                QXD_TRY(blas_axpby(ctx, 1, 0, n, 1.0, 0.0, static_cast<char*>(eb) + i * h32, 1.0, 0.0,
+                                   X64 + open[i] * hb64, st));
+                if (pass == 15) worst = std::max(worst, rels[i]);
             }
-            info->restarts += 1;
-            if (!df) QXD_TRY(blas_axpby(ctx, 0, 1, n, 1.0, 0.0, r64, 0.0, 0.0, rP, st));
-            int ci = 0;
-            QXD_TRY(cg_shifted(ctx, fl, 1, sigma[j], rP, eP, s->nmx - info->iters, std::max(1e-5, 0.5 * s->tol / rel),
-                               &ci, st));
-            info->iters += ci;
-            QXD_TRY(blas_axpby(ctx, 1, 0, n, 1.0, 0.0, eP, 1.0, 0.0, xj, st));
-            if (pass == 15) worst = std::max(worst, rel);
         }
     }
     info->true_relres = worst;
@@ -1306,16 +1292,33 @@ int solve_fgcr_dc_batched(qxd_ctx* ctx, int fl, const qxd_solver* s, const Full&
                 if (verbose()) std::fprintf(stderr, "[qxd dc-batched] GCR stagnated: CGNR inner\n");
             }
         }
-        if (use_cgnr) {
+        if (use_cgnr && Pv == QXD_FP32) {
+            // in lockstep, at most 32 at a time; the fields of the Krylov bases are free here
+            std::vector<double> ctol(B);
+            std::vector<int> it(B, 0);
+            for (int j = 0; j < B; ++j) ctol[j] = rtol[j] >= 1.0 ? 1.0 : std::max(1e-5, 0.5 * s->tol / relres[j]);
+            const int G = std::min(B, 32);
+            void *za, *wa, *ra;
+            QXD_TRY(qxd_ws(ctx, WS_SOLVER + 130, hbP * B, &ra));
+            QXD_TRY(qxd_ws(ctx, WS_SOLVER + 133, 2 * hbP * G, &za));
+            QXD_TRY(qxd_ws(ctx, WS_SOLVER + 134, 2 * hbP * G, &wa));
+            const CgFields work{ra, za, at(za, hbP, G), wa, at(wa, hbP, G)};
+            for (int j = 0; j < B; j += G) {
+                const int nb = std::min(G, B - j);
+                const long long each = s->nmx - info->iters;
+                QXD_TRY(cg_lockstep(ctx, fl, nb, true, nullptr, &ctol[j], at(bP, hbP, j), at(eeP, hbP, j), work, each * nb,
+                                    &it[j], st));
+            }
+            for (int j = 0; j < B; ++j) mx = std::max(mx, 2 * it[j]);
+        } else if (use_cgnr) {
             for (int j = 0; j < B; ++j) {
                 int it = 0;
                 if (rtol[j] >= 1.0) {
                     QXD_CUDA(ctx, cudaMemsetAsync(E + j * hbP, 0, hbP, st));
                     continue;
                 }
-                const double ctol = Pv == QXD_FP64 ? rtol[j] : std::max(1e-5, 0.5 * s->tol / relres[j]);
                 QXD_TRY(cgnr_inner(ctx, fl, Pv, static_cast<char*>(bP) + j * hbP, E + j * hbP, s->nmx - info->iters,
-                                   ctol, &it, st));
+                                   rtol[j], &it, st));
                 mx = std::max(mx, 2 * it);
             }
         }
