@@ -1,10 +1,10 @@
 // Second half of Dhat with the inner products of a GCR step fused into its epilogue
 // (Sec. 2.3 operator; the solver of Sec. 4.4).
 //
-//   w = A_ee r - H_eo t,   t = A_oo^-1 H_oe r  (the first half, an ordinary launch)
+//   w = A_ee r - H_eo t - shift r,   t = A_oo^-1 H_oe r  (the first half, an ordinary launch)
 //
-// The GCR step that applies Dhat to its direction r (the current residual, when the
-// solve has no preconditioner) next needs <W_j, w> for the K earlier basis fields,
+// The solver that applies Dhat to its direction r (the current residual of GCR, or the last
+// vector of a shifted power basis) next needs <W_j, w> for the K earlier basis fields,
 // <r, w> and |w|^2.  Here the thread that has just formed w(x) reads W_j(x) and
 // accumulates them, so the step saves the separate pass that would read w, r and
 // every W_j once more.  FP32 fields, one right-hand side, no gamma5 flags.
@@ -39,7 +39,7 @@ __device__ __forceinline__ void dot_site(const cplx<float> x[12], const cplx<flo
 constexpr int kDotsFlush = 8;
 
 template <int K>
-__global__ void __launch_bounds__(kRedThreads, 2) k_hop_dots(Geo g, HopDev a, MultiPtr W, RedOut o) {
+__global__ void __launch_bounds__(kRedThreads, 2) k_hop_dots(Geo g, HopDev a, float shift, MultiPtr W, RedOut o) {
     constexpr int NC = 2 * K + 4;
     __shared__ double vs[NC][kRedThreads];
     float fa[NC];
@@ -73,11 +73,20 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_hop_dots(Geo g, HopDev a, Mu
 #pragma unroll
             for (int k = 0; k < 12; ++k) acc[k] = c * acc[k] + s[k];
         }
+        {
+            cplx<float> r[12];
+            load_spinor<1>(rin, g.Vh, h, r);
+            if (shift != 0.f) {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) acc[k] = {fmaf(-shift, r[k].re, acc[k].re), fmaf(-shift, r[k].im, acc[k].im)};
+            }
+            dot_site(r, acc, fa[2 * K], fa[2 * K + 1]);
+        }
         store_spinor<1>(out, g.Vh, h, acc);
 #pragma unroll
-        for (int j = 0; j <= K; ++j) {  // the K basis fields, then r
+        for (int j = 0; j < K; ++j) {
             cplx<float> wj[12];
-            load_spinor<1>(j < K ? static_cast<const float4*>(W.p[j]) : rin, g.Vh, h, wj);
+            load_spinor<1>(static_cast<const float4*>(W.p[j]), g.Vh, h, wj);
             dot_site(wj, acc, fa[2 * j], fa[2 * j + 1]);
         }
         float ww = 0.f;
@@ -100,20 +109,57 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_hop_dots(Geo g, HopDev a, Mu
     block_reduce_finish<NC>(v, o);
 }
 
+// r = b - (A_ee e - H_eo t): a restart's residual, with |r|^2 over the finite sites and the
+// number of the others.  Reads the source once instead of copying it, storing Dhat e and
+// subtracting in a pass of its own.
+__global__ void __launch_bounds__(kRedThreads, 2) k_hop_resid(Geo g, HopDev a, const float4* __restrict__ b, RedOut o) {
+    double v[2] = {0.0, 0.0};
+    const float4* in = static_cast<const float4*>(a.in_nb);
+    const float4* ein = static_cast<const float4*>(a.in_self);
+    const int S = gridDim.x * blockDim.x;
+    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.Vh; h += S) {
+        int x[4];
+        site_coords(g, a.pout, h, x);
+        cplx<float> acc[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = {0.f, 0.f};
+        hop_dir<1, 0>(g, a, in, x, h, acc);
+        hop_dir<1, 1>(g, a, in, x, h, acc);
+        hop_dir<1, 2>(g, a, in, x, h, acc);
+        hop_dir<1, 3>(g, a, in, x, h, acc);
+        const float c = (float)(-0.5 * a.c_hop);
+        cplx<float> s[12];
+        load_spinor<1>(ein, g.Vh, h, s);
+        float d[72];
+        load_diag<1>(a.diag, g.Vh, h, d);
+        apply_diag(d, s);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = c * acc[k] + s[k];
+        load_spinor<1>(b, g.Vh, h, s);
+        float n = 0.f;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            acc[k] = s[k] - acc[k];
+            n = fmaf(acc[k].re, acc[k].re, fmaf(acc[k].im, acc[k].im, n));
+        }
+        store_spinor<1>(static_cast<float4*>(a.out), g.Vh, h, acc);
+        if (isfinite(n)) v[0] += n;
+        else v[1] += 1.0;
+    }
+    block_reduce_finish<2>(v, o);
+}
+
 template <int K>
-void launch_k(qxd_ctx* ctx, const HopDev& d, const MultiPtr& W, int slot, cudaStream_t st) {
+void launch_k(qxd_ctx* ctx, const HopDev& d, float shift, const MultiPtr& W, int slot, cudaStream_t st) {
     int nb = wave_blocks(ctx, k_hop_dots<K>, kRedThreads, (size_t)kRedThreads, (size_t)ctx->g.Vh);
     const int cap = kPartials / (2 * K + 4);  // partial sums of every block fit the buffer
     if (nb > cap) nb = cap;
-    k_hop_dots<K><<<nb, kRedThreads, 0, st>>>(ctx->g, d, W, red_out(ctx, slot));
+    k_hop_dots<K><<<nb, kRedThreads, 0, st>>>(ctx->g, d, shift, W, red_out(ctx, slot));
 }
 
 }  // namespace
 
-int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* const* W, int slot, cudaStream_t st) {
-    if (k < 0 || k > kMultiMax) return qxd_fail(ctx, QXD_EARG, "fused hop: at most 8 basis fields");
-    if (a.self_mode != 1 || a.post_mode != 0 || a.nrhs != 1 || a.g5_nb || a.g5_self || a.g5_out)
-        return qxd_fail(ctx, QXD_EARG, "fused hop: only the second half of Dhat, one right-hand side");
+static HopDev hop_dev(qxd_ctx* ctx, int fl, const HopArgs& a) {
     const Geo& g = ctx->g;
     const QxdFlavour& F = ctx->fl[fl];
     const size_t Vh = g.Vh;
@@ -130,21 +176,40 @@ int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* c
     d.diag = F.C32[0] + (size_t)po * 18 * Vh;
     d.diaginv = F.C32[1] + (size_t)po * 18 * Vh;
     d.c_hop = a.c_hop;
+    return d;
+}
+
+int launch_hop_resid(qxd_ctx* ctx, int fl, const HopArgs& a, const void* b, int slot, cudaStream_t st) {
+    const int nb = wave_blocks(ctx, k_hop_resid, kRedThreads, (size_t)kRedThreads, (size_t)ctx->g.Vh);
+    ProfScope prof(ctx, "hop_fp32_resid", (double)ctx->g.Vh * (8 * 56.0 + 288.0 + 96.0 * 4), st);
+    k_hop_resid<<<nb, kRedThreads, 0, st>>>(ctx->g, hop_dev(ctx, fl, a), static_cast<const float4*>(b),
+                                            red_out(ctx, slot));
+    QXD_CUDA(ctx, cudaGetLastError());
+    return QXD_OK;
+}
+
+int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* const* W, double shift, int slot,
+                    cudaStream_t st) {
+    if (k < 0 || k > kMultiMax) return qxd_fail(ctx, QXD_EARG, "fused hop: at most 8 basis fields");
+    if (a.self_mode != 1 || a.post_mode != 0 || a.nrhs != 1 || a.g5_nb || a.g5_self || a.g5_out)
+        return qxd_fail(ctx, QXD_EARG, "fused hop: only the second half of Dhat, one right-hand side");
+    const HopDev d = hop_dev(ctx, fl, a);
+    const size_t Vh = ctx->g.Vh;
     MultiPtr mp{};
     for (int j = 0; j < kMultiMax; ++j) mp.p[j] = W[j < k ? j : 0];
     // algorithmic bytes: the hop with its self term (links 8 x 56, A_ee 288, spinors
     // neighbours + self + output 3 x 96) and the K basis fields
     ProfScope prof(ctx, "hop_fp32_self1_post0_dots", (double)Vh * (8 * 56.0 + 288.0 + 96.0 * (3 + k)), st);
     switch (k) {
-        case 0: launch_k<0>(ctx, d, mp, slot, st); break;
-        case 1: launch_k<1>(ctx, d, mp, slot, st); break;
-        case 2: launch_k<2>(ctx, d, mp, slot, st); break;
-        case 3: launch_k<3>(ctx, d, mp, slot, st); break;
-        case 4: launch_k<4>(ctx, d, mp, slot, st); break;
-        case 5: launch_k<5>(ctx, d, mp, slot, st); break;
-        case 6: launch_k<6>(ctx, d, mp, slot, st); break;
-        case 7: launch_k<7>(ctx, d, mp, slot, st); break;
-        default: launch_k<8>(ctx, d, mp, slot, st); break;
+        case 0: launch_k<0>(ctx, d, (float)shift, mp, slot, st); break;
+        case 1: launch_k<1>(ctx, d, (float)shift, mp, slot, st); break;
+        case 2: launch_k<2>(ctx, d, (float)shift, mp, slot, st); break;
+        case 3: launch_k<3>(ctx, d, (float)shift, mp, slot, st); break;
+        case 4: launch_k<4>(ctx, d, (float)shift, mp, slot, st); break;
+        case 5: launch_k<5>(ctx, d, (float)shift, mp, slot, st); break;
+        case 6: launch_k<6>(ctx, d, (float)shift, mp, slot, st); break;
+        case 7: launch_k<7>(ctx, d, (float)shift, mp, slot, st); break;
+        default: launch_k<8>(ctx, d, (float)shift, mp, slot, st); break;
     }
     QXD_CUDA(ctx, cudaGetLastError());
     return QXD_OK;

@@ -59,8 +59,9 @@ int op_Dhat(qxd_ctx* ctx, int fl, int P, int dagger, const void* in_e, void* out
     return launch_hop(ctx, fl, P, a, st);
 }
 
-int op_Dhat_dots(qxd_ctx* ctx, int fl, const void* in_e, void* out_e, void* tmp_o, int k, const void* const* W,
-                 int slot, cudaStream_t st) {
+// first half of an FP32 Dhat, and the arguments of its second half
+static int dhat_first(qxd_ctx* ctx, int fl, const void* in_e, void* out_e, void* tmp_o, HopArgs* second,
+                      cudaStream_t st) {
     HopArgs a{};
     a.nrhs = 1;
     a.pout = 1;
@@ -77,7 +78,22 @@ int op_Dhat_dots(qxd_ctx* ctx, int fl, const void* in_e, void* out_e, void* tmp_
     a.self_mode = 1;
     a.post_mode = 0;
     a.c_hop = -1.0;
-    return launch_hop_dots(ctx, fl, a, k, W, slot, st);
+    *second = a;
+    return QXD_OK;
+}
+
+int op_Dhat_dots(qxd_ctx* ctx, int fl, const void* in_e, void* out_e, void* tmp_o, int k, const void* const* W,
+                 double shift, int slot, cudaStream_t st) {
+    HopArgs a;
+    QXD_TRY(dhat_first(ctx, fl, in_e, out_e, tmp_o, &a, st));
+    return launch_hop_dots(ctx, fl, a, k, W, shift, slot, st);
+}
+
+int op_Dhat_resid(qxd_ctx* ctx, int fl, const void* b_e, const void* e_e, void* r_e, void* tmp_o, int slot,
+                  cudaStream_t st) {
+    HopArgs a;
+    QXD_TRY(dhat_first(ctx, fl, e_e, r_e, tmp_o, &a, st));
+    return launch_hop_resid(ctx, fl, a, b_e, slot, st);
 }
 
 int op_eo_source(qxd_ctx* ctx, int fl, int P, const Full& r, void* b_e, void* tmp_o, cudaStream_t st, int nrhs) {

@@ -4,6 +4,7 @@
 // the kernels; scalars come back to the host once or twice per iteration.
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstdio>
 #include <cstdlib>
 #include <vector>
@@ -206,9 +207,159 @@ static int precond_into(qxd_ctx* ctx, int fl, int Pv, int Pb, int kind, const vo
     return blas_axpby(ctx, Pv, Pb, n, 1.0, 0.0, ztmp, 0.0, 0.0, z, st);
 }
 
+// Restarted minimal residuals without a preconditioner in FP32, restart lengths up to 16: in
+// exact arithmetic the iterates of GCR(nkv), from a basis that needs no vector update.
+//
+// A cycle forms z_0 = r, z_{k+1} = (Dhat - d) z_k with the inner products <z_j, z_{k+1}> from
+// the operator's second launch (from the ninth step on those with z_0 .. z_{k-9} in a pass of
+// their own), so that the Gram matrix G of z_0 .. z_K is known.  With
+// a_k = Dhat z_k = z_{k+1} + d_k z_k the correction sum_k c_k z_k of minimal residual solves
+// M c = <a, r>, M = (<a_i, a_k>), by a Cholesky factorisation that grows by one row per
+// step; its forward substitution gives the residual norm after every step.  d is the
+// Rayleigh quotient of the first residual: it centres the spectrum, so that the powers stay
+// apart.  A pivot below 1e-7 of its diagonal (the basis is used up at the precision of the
+// sums) ends the cycle there.  The restart takes r = b - Dhat e anew.
+//
+// Why: orthogonalising w_k and updating r in a pass of its own (k_gcr_update, (k + 4) fields)
+// was 16 % of the solve on 32^3x64 C*, and the host looked at every step's numbers before the
+// next was launched.  Solve to 1e-10 there (nkv 8) 72.8 -> 59.7 ms, 56 iterations both; the
+// pivots stay above 1e-5.  From 17 on the powers would end most cycles early: GCR is kept.
+constexpr int kPowerMax = 16;
+static_assert(kPowerMax <= 2 * kMultiMax && kPowerMax * kPowerMax + 5 * kPowerMax + 4 <= kRedSlots, "results of a cycle");
+
+static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b, void* e, int max_iter, double rtol,
+                       int* iters, bool* stagnated, cudaStream_t st) {
+    using C = std::complex<double>;
+    const int nkv = std::max(1, s->nkv);
+    const size_t n = 12ull * ctx->g.Vh;
+    const size_t hb = half_bytes(ctx, QXD_FP32);
+    void *r, *to, *Wb;
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 20, hb, &r));
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 21, hb, &to));
+    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 25, hb * nkv, &Wb));
+    QXD_CUDA(ctx, cudaMemsetAsync(e, 0, hb, st));
+    QXD_TRY(blas_norm2(ctx, QXD_FP32, n, b, 0, st));
+    QXD_TRY(blas_fetch(ctx, 2, st));
+    QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "GCR source"));
+    double rr = ctx->red_host[0];
+    const double target = rtol * rtol * rr;
+    *iters = 0;
+    if (rr == 0.0) return QXD_OK;
+    std::vector<const void*> z(nkv + 1);
+    z[0] = b;
+    for (int k = 0; k < nkv; ++k) z[k + 1] = static_cast<char*>(Wb) + (size_t)k * hb;
+    // results of step k: 2 k + 4 numbers from slot k^2 + 3 k on, in the pinned mirror once event
+    // k % 2 is reached
+    struct Events {
+        cudaEvent_t e[2] = {nullptr, nullptr};
+        ~Events() {
+            for (auto x : e)
+                if (x) cudaEventDestroy(x);
+        }
+    } ev;
+    for (auto& x : ev.e) QXD_CUDA(ctx, cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    std::vector<double> d(nkv, 0.0);
+    double shift = 0.0;
+    bool centred = false;
+    auto launch = [&](int k) -> int {
+        const int slot = k * k + 3 * k;
+        d[k] = shift;
+        const int rest = std::max(0, k - kMultiMax);
+        QXD_TRY(op_Dhat_dots(ctx, fl, z[k], const_cast<void*>(z[k + 1]), to, k - rest, z.data() + rest, shift,
+                             slot + 2 * rest, st));
+        if (rest > 0) QXD_TRY(blas_multi_dot(ctx, QXD_FP32, n, rest, z.data(), z[k + 1], slot, st));
+        QXD_CUDA(ctx, cudaMemcpyAsync(ctx->red_host + slot, ctx->red_result + slot, sizeof(double) * (2 * k + 4),
+                                      cudaMemcpyDeviceToHost, st));
+        QXD_CUDA(ctx, cudaEventRecord(ev.e[k & 1], st));
+        return QXD_OK;
+    };
+    const int m = nkv + 1;
+    std::vector<C> G(m * m), L(nkv * nkv), y(nkv), c(nkv);
+    while (*iters < max_iter) {
+        const int steps = std::min(nkv, max_iter - *iters);
+        const double rr_cycle = rr;
+        G[0] = rr;
+        double drop = 1.0;  // reduction of |r|^2 by the last step
+        int launched = 0, K = 0;
+        bool reached = false, used_up = false;
+        while (K < steps && !reached && !used_up) {
+            if (launched == K) QXD_TRY(launch(launched++));
+            // the next step is queued before this one's numbers are looked at, unless this one may
+            // be the last
+            if (launched < steps && launched == K + 1 && centred && rr * drop > 4.0 * target) QXD_TRY(launch(launched++));
+            QXD_CUDA(ctx, cudaEventSynchronize(ev.e[K & 1]));
+            const int k = K;
+            const double* h = ctx->red_host + k * k + 3 * k;
+            QXD_TRY(status_of_norm(ctx, h[2 * k + 3], "GCR"));
+            for (int j = 0; j <= k; ++j) {
+                G[j * m + k + 1] = C(h[2 * j], h[2 * j + 1]);
+                G[(k + 1) * m + j] = std::conj(G[j * m + k + 1]);
+            }
+            G[(k + 1) * m + k + 1] = h[2 * k + 2];
+            // <z_i, a_k>, the new row of L and the new entry of y
+            auto za = [&](int i) { return G[i * m + k + 1] + d[k] * G[i * m + k]; };
+            double diag = 0.0;
+            for (int i = 0; i <= k; ++i) {
+                C v = std::conj(za(i + 1) + d[i] * za(i));  // <a_k, a_i>
+                if (i == k) diag = v.real();
+                for (int q = 0; q < i; ++q) v -= L[k * nkv + q] * std::conj(L[i * nkv + q]);
+                L[k * nkv + i] = i < k ? v / L[i * nkv + i] : v;
+            }
+            const double pivot = L[k * nkv + k].real();
+            if (!(pivot > 1e-7 * diag) || !std::isfinite(pivot)) {
+                if (k == 0) return qxd_fail(ctx, QXD_EBREAKDOWN, "GCR: |w| = 0");
+                used_up = true;
+                break;
+            }
+            L[k * nkv + k] = std::sqrt(pivot);
+            C v = std::conj(za(0));
+            for (int q = 0; q < k; ++q) v -= L[k * nkv + q] * y[q];
+            y[k] = v / L[k * nkv + k];
+            const double next = rr - std::norm(y[k]);
+            drop = next > 0.0 ? next / rr : 0.0;
+            rr = next;
+            if (!centred) {
+                shift = G[1].real() / G[0].real();
+                centred = true;
+            }
+            ++K;
+            if (verbose())
+                std::fprintf(stderr, "[qxd gcr] it %d k %d pivot %.2e rr %.6e\n", *iters + K, k, pivot / diag, rr);
+            reached = rr <= target;
+        }
+        *iters += launched;
+        for (int k = K - 1; k >= 0; --k) {  // L^+ c = y
+            C v = y[k];
+            for (int q = k + 1; q < K; ++q) v -= std::conj(L[q * nkv + k]) * c[q];
+            c[k] = v / L[k * nkv + k];
+        }
+        double cre[kPowerMax], cim[kPowerMax];
+        for (int k = 0; k < K; ++k) {
+            cre[k] = c[k].real();
+            cim[k] = c[k].imag();
+        }
+        QXD_TRY(blas_multi_axpy(ctx, QXD_FP32, QXD_FP32, n, K, cre, cim, z.data(), e, st));
+        if (reached || *iters >= max_iter) return QXD_OK;
+        QXD_TRY(op_Dhat_resid(ctx, fl, b, e, r, to, 0, st));
+        QXD_TRY(blas_fetch(ctx, 2, st));
+        QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "GCR"));
+        rr = ctx->red_host[0];
+        if (rr <= target) return QXD_OK;
+        // a whole cycle that did not halve the residual norm: restarted GCR stalls
+        if ((K == nkv || used_up) && rr > 0.25 * rr_cycle) {
+            *stagnated = true;
+            return QXD_OK;
+        }
+        z[0] = r;
+    }
+    return QXD_OK;
+}
+
 int fgcr_inner(qxd_ctx* ctx, int fl, int P, const qxd_solver* s, const void* b, void* e, int max_iter,
                double rtol, int* iters, bool* stagnated, cudaStream_t st) {
     *stagnated = false;
+    if (P == QXD_FP32 && s->precond == QXD_PRECOND_NONE && s->nkv <= kPowerMax)
+        return gcr_power32(ctx, fl, s, b, e, max_iter, rtol, iters, stagnated, st);
     const int Pb = P, Pv = vec_prec(P);
     const bool split = Pb != Pv;
     const int nkv = s->nkv < 1 ? 1 : (s->nkv > 64 ? 64 : s->nkv);
@@ -259,7 +410,7 @@ int fgcr_inner(qxd_ctx* ctx, int fl, int P, const qxd_solver* s, const void* b, 
             // own second launch (op_Dhat_dots), which also counts non-finite sites.
             double nonfinite = 0.0;
             if (rz && Pb == QXD_FP32 && k <= kMultiMax) {
-                QXD_TRY(op_Dhat_dots(ctx, fl, Z[k], W[k], to, k, W.data(), 0, st));
+                QXD_TRY(op_Dhat_dots(ctx, fl, Z[k], W[k], to, k, W.data(), 0.0, 0, st));
                 QXD_TRY(blas_fetch(ctx, 2 * k + 4, st));
                 nonfinite = ctx->red_host[2 * k + 3];
             } else {
