@@ -228,6 +228,216 @@ __global__ void __launch_bounds__(256, 1) k_hop_canon(Geo g, CanonDev a, int nrh
     }
 }
 
+// Small lattices: four lanes per site, lane q the two hops of direction q.
+//
+// With a thread per site such a launch is one long chain of instructions on a few warps, and
+// on the FP64 pipe (64 cycles per warp instruction) most of the chip's schedulers have none.
+// Four lanes shorten the chain and fill four times the warps; the launch also lets the next
+// one start early, which loads its links and site-diagonal terms meanwhile.  Measured per
+// call, one thread -> four lanes (us): Dhat 8^4 FP32 12.4 -> 6.4 (then bound by the host), FP64
+// 84 -> 48; D_w 4 x 4 x 8 x 8 FP64 41 -> 15.  The exchanges and the site-diagonal term done
+// twice cost more than that beyond about 8192 sites in FP32 (Dhat on 8 x 8 x 16 x 16 with two
+// right-hand sides 12.4 -> 13.0) and 4096 in FP64 (81 against 84 us there, 88 against 84 at 8192).
+//
+// A lane forms the half-spinors of its direction's forward and backward hop; their sums and
+// differences give its share of the upper and lower spins.  Two exchanges leave the upper
+// chiral block in lanes 0, 1 and the lower one in lanes 2, 3, both lanes of a pair apply the
+// block's 6 x 6 site-diagonal term and each stores three of the six components.
+constexpr int kQuadThreads = 64;
+
+template <typename R>
+__device__ __forceinline__ cplx<R> sel(bool c, cplx<R> a, cplx<R> b) {
+    return {c ? a.re : b.re, c ? a.im : b.im};
+}
+template <typename R>
+__device__ __forceinline__ cplx<R> shfl_x(cplx<R> a, int m) {
+    return {__shfl_xor_sync(0xffffffffu, a.re, m), __shfl_xor_sync(0xffffffffu, a.im, m)};
+}
+
+template <int P, int MODE>
+__global__ void __launch_bounds__(kQuadThreads) k_hop_quad(Geo g, CanonDev a, int nrhs) {
+    using R = typename Prec<P>::real;
+    using CH = typename Prec<P>::chunk;
+    using C = cplx<R>;
+    // the next launch of the stream may begin: it reads links and site-diagonal terms (which
+    // no kernel that allows this writes) and waits before it touches a field
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int sites = MODE == kDw ? (int)g.V : g.Vh;
+    const int Vh = g.Vh;
+    const int rhs = blockIdx.x % nrhs;
+    const int site = (blockIdx.x / nrhs) * (kQuadThreads / 4) + (threadIdx.x >> 2);
+    const bool live = site < sites;
+    const int i = live ? site : sites - 1;  // every lane takes part in the exchanges
+    const int q = threadIdx.x & 3;
+    int x[4], p, h;
+    if constexpr (MODE == kDw) {
+        int r = i;
+        x[3] = r % g.N[3];
+        r /= g.N[3];
+        x[2] = r % g.N[2];
+        r /= g.N[2];
+        x[1] = r % g.N[1];
+        x[0] = r / g.N[1];
+        p = (x[0] + x[1] + x[2] + x[3]) & 1;
+        h = i >> 1;
+    } else {
+        p = MODE == kDhat1 ? 1 : 0;
+        h = i;
+        site_coords(g, p, h, x);
+    }
+    const int yf = q == 0 ? neighbour_lex(g, x, 0, +1) : q == 1 ? neighbour_lex(g, x, 1, +1) : q == 2 ? neighbour_lex(g, x, 2, +1) : neighbour_lex(g, x, 3, +1);
+    const int yb = q == 0 ? neighbour_lex(g, x, 0, -1) : q == 1 ? neighbour_lex(g, x, 1, -1) : q == 2 ? neighbour_lex(g, x, 2, -1) : neighbour_lex(g, x, 3, -1);
+    Mat3<R> mf, mb;
+    cplx<float> zf, zb;
+    if constexpr (P == 0) {
+        load_link64(a.V64 + (size_t)p * 36 * Vh, Vh, q, h, mf);
+        load_link64(a.V64 + (size_t)(1 - p) * 36 * Vh, Vh, q, yb >> 1, mb);
+    } else {
+        load_link32(a.U32 + (size_t)p * 12 * Vh, a.Z32 + (size_t)p * 2 * Vh, Vh, q, h, mf, zf);
+        load_link32(a.U32 + (size_t)(1 - p) * 12 * Vh, a.Z32 + (size_t)(1 - p) * 2 * Vh, Vh, q, yb >> 1, mb, zb);
+    }
+    // the lane's 6 x 6 block (block q / 2)
+    constexpr int NB = P == 0 ? 18 : 9;
+    R d[36];
+    {
+        const CH* D = static_cast<const CH*>(a.diag) + ((size_t)p * 2 + (q >> 1)) * NB * Vh + h;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            const CH v = QXD_LDG(D + (size_t)k * Vh);
+            if constexpr (P == 0) {
+                d[2 * k] = v.x;
+                d[2 * k + 1] = v.y;
+            } else {
+                d[4 * k] = v.x;
+                d[4 * k + 1] = v.y;
+                d[4 * k + 2] = v.z;
+                d[4 * k + 3] = v.w;
+            }
+        }
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const size_t canon = (size_t)rhs * sites * 24, inner = (size_t)rhs * Prec<P>::nchunk * Vh;
+    C sf[12], sb[12];
+    if constexpr (MODE == kDhat2) {
+        const CH* t = static_cast<const CH*>(a.nb) + inner;
+        load_spinor<P>(t, Vh, yf >> 1, sf);
+        load_spinor<P>(t, Vh, yb >> 1, sb);
+    } else {
+        const R* f = static_cast<const R*>(a.nb) + canon;
+        load_canon<P, false>(f, MODE == kDw ? yf : yf >> 1, sf);
+        load_canon<P, false>(f, MODE == kDw ? yb : yb >> 1, sb);
+    }
+    const bool dg = a.dagger != 0;
+    if (MODE == kDhat1 && dg) {
+#pragma unroll
+        for (int k = 6; k < 12; ++k) {
+            sf[k] = -sf[k];
+            sb[k] = -sb[k];
+        }
+    }
+    // projections s_0 +- c_0 s_p0, s_1 +- c_1 s_p1: p = (2, 3) for directions 0, 3, (3, 2) for
+    // 1, 2; c = 1 or i, c_1 with the opposite sign for 2, 3
+    const bool imag = q & 1, swap = q == 1 || q == 2;
+    const R s1 = q >= 2 ? R(-1) : R(1);
+    Half<R> hf, hb, rf, rb;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        C b0 = sel(swap, sf[9 + c], sf[6 + c]), b1 = sel(swap, sf[6 + c], sf[9 + c]);
+        b0 = sel(imag, times_i(b0), b0);
+        b1 = s1 * sel(imag, times_i(b1), b1);
+        hf.a[0][c] = sf[c] + b0;
+        hf.a[1][c] = sf[3 + c] + b1;
+        b0 = sel(swap, sb[9 + c], sb[6 + c]), b1 = sel(swap, sb[6 + c], sb[9 + c]);
+        b0 = sel(imag, times_i(b0), b0);
+        b1 = s1 * sel(imag, times_i(b1), b1);
+        hb.a[0][c] = sb[c] - b0;
+        hb.a[1][c] = sb[3 + c] - b1;
+    }
+    mul_half<false>(mf, hf, rf);
+    mul_half<true>(mb, hb, rb);
+    if constexpr (P != 0) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                rf.a[s][c] = zf * rf.a[s][c];
+                rb.a[s][c] = cmul_conj(zb, rb.a[s][c]);
+            }
+    }
+    // upper spins get the sum, spin p0 c_0^* and spin p1 c_1^* times the difference; lanes 0, 1
+    // keep the upper block, 2, 3 the lower one
+    C v[6];
+    const bool low = q >= 2;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const C u0 = rf.a[0][c] + rb.a[0][c], u1 = rf.a[1][c] + rb.a[1][c];
+        C e0 = rf.a[0][c] - rb.a[0][c], e1 = s1 * (rf.a[1][c] - rb.a[1][c]);
+        e0 = sel(imag, -times_i(e0), e0);
+        e1 = sel(imag, -times_i(e1), e1);
+        const C l2 = sel(swap, e1, e0), l3 = sel(swap, e0, e1);
+        const C k0 = sel(low, l2, u0), k1 = sel(low, l3, u1);
+        v[c] = k0 + shfl_x(sel(low, u0, l2), 2);
+        v[3 + c] = k1 + shfl_x(sel(low, u1, l3), 2);
+    }
+    const R hc = MODE == kDhat2 ? R(0.5) : R(-0.5);  // -1/2 times the sign of the hopping term
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = hc * (v[k] + shfl_x(v[k], 1));
+    C o[6];
+    if constexpr (MODE == kDhat1) {
+        herm6_mul(d, v, o);
+    } else {
+        const R* f = static_cast<const R*>(a.self) + canon + (size_t)i * 24 + 12 * (q >> 1);
+        C s[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) s[k] = {f[2 * k], f[2 * k + 1]};
+        if (MODE == kDhat2 && dg && low) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) s[k] = -s[k];
+        }
+        herm6_mul(d, s, o);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) o[k] = v[k] + o[k];
+        if (MODE == kDhat2 && dg && low) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) o[k] = -o[k];
+        }
+    }
+    // both lanes of a pair have read the site's own input by now (in place: before either writes)
+    __syncwarp();
+    if (!live) return;
+    const bool odd = q & 1;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const C w = sel(odd, o[3 + k], o[k]);
+        if constexpr (MODE == kDhat1) {
+            const int m = 3 * q + k;  // component of the internal field
+            if constexpr (P == 0) static_cast<double2*>(a.out)[inner + (size_t)m * Vh + h] = make_double2(w.re, w.im);
+            else reinterpret_cast<float2*>(static_cast<float4*>(a.out) + inner + (size_t)(m >> 1) * Vh + h)[m & 1] = make_float2(w.re, w.im);
+        } else {
+            R* f = static_cast<R*>(a.out) + canon + (size_t)i * 24 + 6 * q + 2 * k;
+            f[0] = w.re;
+            f[1] = w.im;
+        }
+    }
+}
+
+// site and right-hand-side products up to which four lanes per site are the faster
+constexpr long long quad_sites(int prec) { return prec == QXD_FP64 ? 4096 : 8192; }
+
+template <int P, int MODE>
+cudaError_t launch_quad(const Geo& g, const CanonDev& a, int nrhs, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(nblocks(MODE == kDw ? g.V : g.Vh, kQuadThreads / 4) * nrhs));
+    cfg.blockDim = dim3(kQuadThreads);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_hop_quad<P, MODE>, g, a, nrhs);
+}
+
 template <int MODE>
 int launch_canon(qxd_ctx* ctx, int fl, int prec, const void* nb, const void* self, void* out, int dagger, int nrhs,
                  cudaStream_t st) {
@@ -242,13 +452,18 @@ int launch_canon(qxd_ctx* ctx, int fl, int prec, const void* nb, const void* sel
     char name[48];
     std::snprintf(name, sizeof name, "hop_%s_%s%s", prec == QXD_FP64 ? "fp64" : prec == QXD_FP32 ? "fp32" : "bf16", mode,
                   nrhs > 1 ? "_mrhs" : "");
-    // D_w of several right-hand sides goes over the sites in two launches (the first and the
-    // second half), as many as the half-lattice kernels take; one right-hand side in one
+    // D_w of several right-hand sides on a large lattice goes over the sites in two launches
+    // (the first and the second half), as many as the half-lattice kernels take
     const int sites = MODE == kDw ? (int)g.V : g.Vh;
-    const int parts = MODE == kDw && nrhs > 1 ? 2 : 1;
+    const int parts = MODE == kDw && nrhs > 1 && (long long)sites * nrhs > (1 << 20) ? 2 : 1;
     for (int k = 0; k < parts; ++k) {
         const int first = k * (sites / parts), end = k + 1 == parts ? sites : (k + 1) * (sites / parts);
         ProfScope prof(ctx, name, (double)g.Vh * ((MODE == kDw ? link + 2 * dg : link + dg) + per * nrhs) / parts, st);
+        if (prec != QXD_BF16 && (long long)sites * nrhs <= quad_sites(prec)) {
+            const cudaError_t e = prec == QXD_FP64 ? launch_quad<0, MODE>(g, a, nrhs, st) : launch_quad<1, MODE>(g, a, nrhs, st);
+            QXD_CUDA(ctx, e);
+            continue;
+        }
         const int grid = nblocks(end - first, kCanonThreads) * nrhs;
         if (prec == QXD_FP64) k_hop_canon<0, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs, first, end);
         else if (prec == QXD_FP32) k_hop_canon<1, MODE><<<grid, kCanonThreads, 0, st>>>(g, a, nrhs, first, end);
