@@ -38,10 +38,11 @@ __device__ __forceinline__ void dot_site(const cplx<float> x[12], const cplx<flo
 // shared memory (the FP64 accumulators would not fit the registers of the hop)
 constexpr int kDotsFlush = 8;
 
-template <int K>
-__global__ void __launch_bounds__(kRedThreads, 2) k_hop_dots(Geo g, HopDev a, float shift, MultiPtr W, RedOut o) {
+// T threads per block: 64 where blocks of 256 would leave most of the chip without one
+template <int K, int T>
+__global__ void __launch_bounds__(T, 512 / T) k_hop_dots(Geo g, HopDev a, float shift, MultiPtr W, RedOut o) {
     constexpr int NC = 2 * K + 4;
-    __shared__ double vs[NC][kRedThreads];
+    __shared__ double vs[NC][T];
     float fa[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -103,10 +104,9 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_hop_dots(Geo g, HopDev a, fl
             }
         }
     }
-    double v[NC];
 #pragma unroll
-    for (int q = 0; q < NC; ++q) v[q] = vs[q][threadIdx.x] + fa[q];
-    block_reduce_finish<NC>(v, o);
+    for (int q = 0; q < NC; ++q) vs[q][threadIdx.x] += fa[q];
+    smem_reduce_finish<NC, T>(vs, o);
 }
 
 // r = b - (A_ee e - H_eo t): a restart's residual, with |r|^2 over the finite sites and the
@@ -149,12 +149,19 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_hop_resid(Geo g, HopDev a, c
     block_reduce_finish<2>(v, o);
 }
 
-template <int K>
-void launch_k(qxd_ctx* ctx, const HopDev& d, float shift, const MultiPtr& W, int slot, cudaStream_t st) {
-    int nb = wave_blocks(ctx, k_hop_dots<K>, kRedThreads, (size_t)kRedThreads, (size_t)ctx->g.Vh);
+template <int K, int T>
+void launch_kt(qxd_ctx* ctx, const HopDev& d, float shift, const MultiPtr& W, int slot, cudaStream_t st) {
+    int nb = wave_blocks(ctx, k_hop_dots<K, T>, T, (size_t)T, (size_t)ctx->g.Vh);
     const int cap = kPartials / (2 * K + 4);  // partial sums of every block fit the buffer
     if (nb > cap) nb = cap;
-    k_hop_dots<K><<<nb, kRedThreads, 0, st>>>(ctx->g, d, shift, W, red_out(ctx, slot));
+    k_hop_dots<K, T><<<nb, T, 0, st>>>(ctx->g, d, shift, W, red_out(ctx, slot));
+}
+
+template <int K>
+void launch_k(qxd_ctx* ctx, const HopDev& d, float shift, const MultiPtr& W, int slot, cudaStream_t st) {
+    // less than one wave of 256-thread blocks (two per SM)
+    if (ctx->g.Vh < 512 * ctx->nsm) launch_kt<K, 64>(ctx, d, shift, W, slot, st);
+    else launch_kt<K, kRedThreads>(ctx, d, shift, W, slot, st);
 }
 
 }  // namespace

@@ -50,53 +50,71 @@ struct RedOut {
 
 static RedOut red_out(qxd_ctx* ctx, int slot) { return RedOut{ctx->red_partials, ctx->red_ticket, ctx->red_result + slot}; }
 
-template <int NC>
-__device__ void block_reduce_finish(double v[NC], const RedOut& o) {
-    __shared__ double sh[NC][kRedThreads / 32];
+// Sums of NC numbers over the grid from the T threads' values in shared memory vs[c][thread].
+// A warp's FP64 addition holds its scheduler for 64 cycles, so each number is summed by one
+// group of warps (32 lanes x a few values, five shuffles) instead of by every warp, and the
+// last block sums the numbers' partials side by side: with 20 numbers on 42 blocks the whole
+// launch took 35 us when every warp shuffled every number and the last block went through them
+// one after the other, 22 us so (k_hop_dots on 8 x 28 x 12 x 8; k_multi_dot with eight fields
+// 18 -> 10 us).
+template <int NC, int T>
+__device__ void smem_reduce_finish(double (*vs)[T], const RedOut& o) {
+    constexpr int NW = T / 32;
+    constexpr int WP = NC >= NW ? 1 : NC > NW / 2 ? 1 : NC > NW / 4 ? 2 : NC > NW / 8 ? 4 : 8;  // warps of a number
+    __shared__ double sub[NC][WP];
     __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int s = warp % WP;
+    __syncthreads();
+    for (int c = warp / WP; c < NC; c += NW / WP) {
+        double x = 0.0;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        double x = v[c];
+        for (int k = 0; k < NW / WP; ++k) x += vs[c][lane + 32 * (s + WP * k)];
 #pragma unroll
-        for (int s = 16; s > 0; s >>= 1) x += __shfl_down_sync(0xffffffffu, x, s);
-        if (lane == 0) sh[c][warp] = x;
+        for (int m = 16; m > 0; m >>= 1) x += __shfl_down_sync(0xffffffffu, x, m);
+        if (lane == 0) sub[c][s] = x;
     }
     __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            double x = lane < kRedThreads / 32 ? sh[c][lane] : 0.0;
-#pragma unroll
-            for (int s = 16; s > 0; s >>= 1) x += __shfl_down_sync(0xffffffffu, x, s);
-            if (lane == 0) o.partials[(size_t)c * gridDim.x + blockIdx.x] = x;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < NC) {
+        double x = sub[threadIdx.x][0];
+        for (int k = 1; k < WP; ++k) x += sub[threadIdx.x][k];
+        o.partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = x;
         __threadfence();
-        last = atomicAdd(o.ticket, 1u) == gridDim.x - 1;
     }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(o.ticket, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
     const int nb = gridDim.x;
-    for (int c = 0; c < NC; ++c) {
+    for (int c = warp / WP; c < NC; c += NW / WP) {
+        const double* part = o.partials + (size_t)c * nb;
         double x = 0.0;
-        for (int b = threadIdx.x; b < nb; b += blockDim.x) x += __ldcg(o.partials + (size_t)c * nb + b);
+        for (int b = lane + 32 * s; b < nb; b += 4 * 32 * WP) {
+            double y[4];
 #pragma unroll
-        for (int s = 16; s > 0; s >>= 1) x += __shfl_down_sync(0xffffffffu, x, s);
-        __syncthreads();
-        if (lane == 0) sh[0][warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            x = lane < kRedThreads / 32 ? sh[0][lane] : 0.0;
-#pragma unroll
-            for (int s = 16; s > 0; s >>= 1) x += __shfl_down_sync(0xffffffffu, x, s);
-            if (lane == 0) o.result[c] = x;
+            for (int k = 0; k < 4; ++k) y[k] = b + k * 32 * WP < nb ? __ldcg(part + b + k * 32 * WP) : 0.0;
+            x += (y[0] + y[1]) + (y[2] + y[3]);
         }
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) x += __shfl_down_sync(0xffffffffu, x, m);
+        if (lane == 0) sub[c][s] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x < NC) {
+        double x = sub[threadIdx.x][0];
+        for (int k = 1; k < WP; ++k) x += sub[threadIdx.x][k];
+        o.result[threadIdx.x] = x;
     }
     if (threadIdx.x == 0) *o.ticket = 0u;
+}
+
+template <int NC>
+__device__ void block_reduce_finish(double v[NC], const RedOut& o) {
+    __shared__ double vs[NC][kRedThreads];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) vs[c][threadIdx.x] = v[c];
+    smem_reduce_finish<NC, kRedThreads>(vs, o);
 }
 
 }  // namespace qxd
