@@ -48,7 +48,8 @@ __device__ __forceinline__ void ld32(const float* p, float v[8]) {
 __device__ __forceinline__ void ld32(const double* p, double v[4]) {
     asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
 }
-// of an array that the same launch writes (each thread its own site): not the read-only path
+// of an array that is written while the launch exists (by itself, each thread its own site, or by
+// the kernel before an early launch): not the read-only path
 __device__ __forceinline__ void ld32_rw(const float* p, float v[8]) {
     asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
@@ -254,6 +255,22 @@ __device__ __forceinline__ cplx<R> shfl_x(cplx<R> a, int m) {
     return {__shfl_xor_sync(0xffffffffu, a.re, m), __shfl_xor_sync(0xffffffffu, a.im, m)};
 }
 
+__device__ __forceinline__ void load_inner_rw(const float4* b, int Vh, int h, cplx<float> s[12]) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const float4 v = b[(size_t)k * Vh + h];
+        s[2 * k] = {v.x, v.y};
+        s[2 * k + 1] = {v.z, v.w};
+    }
+}
+__device__ __forceinline__ void load_inner_rw(const double2* b, int Vh, int h, cplx<double> s[12]) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const double2 v = b[(size_t)k * Vh + h];
+        s[k] = {v.x, v.y};
+    }
+}
+
 template <int P, int MODE>
 __global__ void __launch_bounds__(kQuadThreads) k_hop_quad(Geo g, CanonDev a, int nrhs) {
     using R = typename Prec<P>::real;
@@ -318,14 +335,15 @@ __global__ void __launch_bounds__(kQuadThreads) k_hop_quad(Geo g, CanonDev a, in
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const size_t canon = (size_t)rhs * sites * 24, inner = (size_t)rhs * Prec<P>::nchunk * Vh;
     C sf[12], sb[12];
+    // not by the read-only path: a kernel that writes the field may run until the wait above
     if constexpr (MODE == kDhat2) {
         const CH* t = static_cast<const CH*>(a.nb) + inner;
-        load_spinor<P>(t, Vh, yf >> 1, sf);
-        load_spinor<P>(t, Vh, yb >> 1, sb);
+        load_inner_rw(t, Vh, yf >> 1, sf);
+        load_inner_rw(t, Vh, yb >> 1, sb);
     } else {
         const R* f = static_cast<const R*>(a.nb) + canon;
-        load_canon<P, false>(f, MODE == kDw ? yf : yf >> 1, sf);
-        load_canon<P, false>(f, MODE == kDw ? yb : yb >> 1, sb);
+        load_canon<P, true>(f, MODE == kDw ? yf : yf >> 1, sf);
+        load_canon<P, true>(f, MODE == kDw ? yb : yb >> 1, sb);
     }
     const bool dg = a.dagger != 0;
     if (MODE == kDhat1 && dg) {
