@@ -464,6 +464,7 @@ int cg_lockstep(qxd_ctx* ctx, int fl, int B, bool normal, const double* sigma, c
         else if (chunk - looked > 1) rc = look(looked++ & 1);
     }
     while (rc == QXD_OK && looked < chunk) rc = look(looked++ & 1);
+    if (rc != QXD_OK) cudaStreamSynchronize(st);  // what is still queued uses the workspaces
     for (auto& x : ev2)
         if (x) cudaEventDestroy(x);
     for (int j = 0; j < B; ++j) iters[j] = done[j];

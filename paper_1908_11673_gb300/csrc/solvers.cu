@@ -251,15 +251,18 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
     // results of step k: 2 k + 4 numbers from slot k^2 + 3 k on, in the pinned mirror once event
     // k % 2 is reached
     struct Events {
+        cudaStream_t st;
+        bool ok = false;
         cudaEvent_t e[2] = {nullptr, nullptr};
         ~Events() {
+            if (!ok) cudaStreamSynchronize(st);  // a step that is still queued uses the workspaces
             for (auto x : e)
                 if (x) cudaEventDestroy(x);
         }
-    } ev;
+    } ev{st};
     for (auto& x : ev.e) QXD_CUDA(ctx, cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
     std::vector<double> d(nkv, 0.0);
-    double shift = 0.0;
+    double shift = 0.0;  // an FP32 number, as the kernel applies it
     bool centred = false;
     auto launch = [&](int k) -> int {
         const int slot = k * k + 3 * k;
@@ -276,11 +279,10 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
     const int m = nkv + 1;
     std::vector<C> G(m * m), L(nkv * nkv), y(nkv), c(nkv);
     while (*iters < max_iter) {
-        const int steps = std::min(nkv, max_iter - *iters);
         const double rr_cycle = rr;
         G[0] = rr;
         double drop = 1.0;  // reduction of |r|^2 by the last step
-        int launched = 0, K = 0;
+        int steps = std::min(nkv, max_iter - *iters), launched = 0, K = 0;
         bool reached = false, used_up = false;
         while (K < steps && !reached && !used_up) {
             if (launched == K) QXD_TRY(launch(launched++));
@@ -305,8 +307,18 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
                 for (int q = 0; q < i; ++q) v -= L[k * nkv + q] * std::conj(L[i * nkv + q]);
                 L[k * nkv + i] = i < k ? v / L[i * nkv + i] : v;
             }
+            // z_1 close to -d z_0 (a residual almost in the kernel): |Dhat z_0|^2 is lost in the
+            // difference, from here on the powers are taken without a shift
+            const double scale = h[2 * k + 2] + d[k] * d[k] * G[k * m + k].real();
+            if (k == 0 && d[0] != 0.0 && !(diag > 1e-5 * scale)) {
+                shift = 0.0;
+                *iters += launched;
+                steps = std::min(nkv, max_iter - *iters);
+                launched = 0;
+                continue;
+            }
             const double pivot = L[k * nkv + k].real();
-            if (!(pivot > 1e-7 * diag) || !std::isfinite(pivot)) {
+            if (!(pivot > 1e-7 * diag) || !(diag > 1e-6 * scale) || !std::isfinite(pivot)) {
                 if (k == 0) return qxd_fail(ctx, QXD_EBREAKDOWN, "GCR: |w| = 0");
                 used_up = true;
                 break;
@@ -319,7 +331,7 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
             drop = next > 0.0 ? next / rr : 0.0;
             rr = next;
             if (!centred) {
-                shift = G[1].real() / G[0].real();
+                shift = (double)(float)(G[1].real() / G[0].real());
                 centred = true;
             }
             ++K;
@@ -338,20 +350,20 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
             cre[k] = c[k].real();
             cim[k] = c[k].imag();
         }
-        QXD_TRY(blas_multi_axpy(ctx, QXD_FP32, QXD_FP32, n, K, cre, cim, z.data(), e, st));
-        if (reached || *iters >= max_iter) return QXD_OK;
+        if (K > 0) QXD_TRY(blas_multi_axpy(ctx, QXD_FP32, QXD_FP32, n, K, cre, cim, z.data(), e, st));
+        ev.ok = reached || *iters >= max_iter;
+        if (ev.ok) return QXD_OK;
         QXD_TRY(op_Dhat_resid(ctx, fl, b, e, r, to, 0, st));
         QXD_TRY(blas_fetch(ctx, 2, st));
         QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "GCR"));
         rr = ctx->red_host[0];
-        if (rr <= target) return QXD_OK;
         // a whole cycle that did not halve the residual norm: restarted GCR stalls
-        if ((K == nkv || used_up) && rr > 0.25 * rr_cycle) {
-            *stagnated = true;
-            return QXD_OK;
-        }
+        *stagnated = rr > target && (K == nkv || used_up) && rr > 0.25 * rr_cycle;
+        ev.ok = rr <= target || *stagnated;
+        if (ev.ok) return QXD_OK;
         z[0] = r;
     }
+    ev.ok = true;
     return QXD_OK;
 }
 

@@ -3,16 +3,17 @@
 Restart lengths on both sides of where the inner products split (8) and of where the
 power basis ends (16), one step per cycle, a budget that ends within a cycle, and an
 operator proportional to the identity up to the site-diagonal term (a basis that is used
-up after a few steps).  Solutions are held to the requested true residual with the FP64
+up after a few steps), a residual almost in the operator's kernel.  Solutions are held to the requested true residual with the FP64
 oracle; the iteration count of a restart length is that of GCR, whose iterates the method
 reproduces in exact arithmetic, to within one cycle per outer step.
 """
 import numpy as np
 import pytest
 
+from oracle import DiracOperator, Flavour, GaugeField, Geometry
 from oracle.solvers import gcr
 from paper_1908_11673_gb300 import workload
-from tests.gpu_helpers import setup
+from tests.gpu_helpers import need_gpu, setup
 
 pytestmark = pytest.mark.gpu
 
@@ -50,4 +51,30 @@ def test_basis_that_is_used_up(nkv):
     zero = np.zeros_like(eta)
     ctx.solve(0, zero, psi, nkv=nkv, inner=qxd.FP32, tol=1e-10)
     assert not psi.any()
+    ctx.close()
+
+
+@pytest.mark.parametrize("nkv", [1, 2])
+def test_residual_almost_in_the_kernel(nkv):
+    # Free field, bare mass m0 = 5e-4.  On the even sites Dhat multiplies a constant spinor by
+    # about 2 m0 and the mode (-1)^(x2 + x3), which the hopping term annihilates, by 1/(2 kappa).
+    # The first cycle takes the second mode away and centres the powers on it; for what is
+    # left |Dhat r|^2 is below the rounding of |d r|^2.
+    kappa = 0.5 / (4 + 5e-4)
+    L, zero = (8, 8, 8, 8), (0.0, 0.0, 0.0, 0.0)
+    qxd = need_gpu()
+    geom = Geometry(L, 0, zero)
+    U = np.broadcast_to(np.eye(3, dtype=complex), (geom.V, 4, 3, 3)).copy()
+    A = np.zeros((geom.V, 4))
+    op = DiracOperator(GaugeField(geom, U, A, 6.0), Flavour(4, kappa, 1.0, 1.0))
+    ctx = qxd.Context(L, 0, zero)
+    ctx.set_links(U, A, 6.0)
+    ctx.set_clover(0, 4, kappa, 1.0, 1.0)
+    x = np.stack(np.unravel_index(np.arange(geom.V), L))
+    lo = np.random.default_rng(3).standard_normal((4, 3))
+    eta = (1 - x.sum(0) % 2)[:, None, None] * (((-1.0) ** (x[2] + x[3]))[:, None, None] + 0.1 * lo) + 0j
+    psi = np.empty_like(eta)
+    info = ctx.solve(0, eta, psi, nkv=nkv, inner=qxd.FP32, tol=1e-5)
+    assert np.linalg.norm(eta - op.apply(psi)) <= 1e-5 * np.linalg.norm(eta)
+    assert info.iters <= 20
     ctx.close()
