@@ -533,10 +533,11 @@ static int sap_blocks(qxd_ctx* ctx, int fl, SapDev& a, int nblk, cudaStream_t st
     QxdFlavour& F = ctx->fl[fl];
     const char* env = std::getenv("QXD_SAP_BLOCKS");
     if (env && env[0] == '0') return QXD_OK;
+    // a captured graph may outlive the copies
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return QXD_OK;
     if (!F.sap && !F.sap_off) {
         void* p;
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return QXD_OK;
         if (!dev_alloc(ctx, &p, sizeof(SapBlock) * (size_t)nblk)) {
             F.sap_off = true;
             return QXD_OK;
