@@ -32,8 +32,11 @@ int qxd_fail(qxd_ctx* ctx, int code, const std::string& msg) {
 // qxd_set_links kept for flavours not set again since and the SAP copies (the sweeps do
 // without) are given back first.
 bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes) {
-    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaSuccess) return true;
     cudaGetLastError();
+    *p = nullptr;
+    if (e != cudaErrorMemoryAllocation) return false;
     for (auto& F : ctx->fl) {
         if (!F.set && !F.building) free_fields(F);
         if (F.sap) {
@@ -46,6 +49,13 @@ bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes) {
     cudaGetLastError();
     *p = nullptr;
     return false;
+}
+
+void qxd_ws_free(qxd_ctx* ctx, int slot) {
+    if (slot < 0 || slot >= (int)ctx->ws_ptr.size()) return;
+    cudaFree(ctx->ws_ptr[slot]);
+    ctx->ws_ptr[slot] = nullptr;
+    ctx->ws_size[slot] = 0;
 }
 
 int qxd_ws(qxd_ctx* ctx, int slot, size_t bytes, void** out) {

@@ -476,10 +476,15 @@ static int launch_clover(qxd_ctx* ctx, int fl, cudaStream_t st) {
     const int N0 = g.N[0];
     int S = (int)std::min<size_t>(N0, (512ull << 20) / per);  // slices of a slab
     if (S < N0) S = std::max(S - 1, 1);                       // room for the slice before it
-    const bool whole = S + 1 >= N0;
-    sl.slots = whole ? N0 : S + 1;
-    void* t;
-    QXD_TRY(qxd_ws(ctx, WS_CLOVER, per * sl.slots, &t));
+    bool whole = false;
+    void* t = nullptr;
+    for (;; S = (S + 1) / 2) {  // smaller slabs where there is no memory for them
+        whole = S + 1 >= N0;
+        sl.slots = whole ? N0 : S + 1;
+        const int rc = qxd_ws(ctx, WS_CLOVER, per * sl.slots, &t);
+        if (rc == QXD_OK) break;
+        if (S == 1) return rc;
+    }
     sl.t = static_cast<double*>(t);
     ProfScope prof(ctx, "set_clover", (double)g.V * (4 * 144 + 4 * 8 + 2 * (576 + 288)), st);
     for (int a = 0; a < N0; a += whole ? N0 : S) {

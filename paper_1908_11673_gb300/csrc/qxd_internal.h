@@ -111,6 +111,7 @@ int qxd_fail(qxd_ctx* ctx, int code, const std::string& msg);
 
 // workspace slot `slot` with at least `bytes` bytes (device memory)
 int qxd_ws(qxd_ctx* ctx, int slot, size_t bytes, void** out);
+void qxd_ws_free(qxd_ctx* ctx, int slot);
 
 // device memory for the context (api.cu); false if there is none
 bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes);

@@ -1029,15 +1029,18 @@ int solve_mscg(qxd_ctx* ctx, int fl, int ns, const double* sigma, const qxd_solv
     // them); groups of at most kRefineBytes per field block, so that the workspace stays small
     // on large lattices
     const size_t h32 = half_bytes(ctx, QXD_FP32);
-    const int group = (int)std::max<size_t>(1, std::min<size_t>(ns, kRefineBytes / h32));
+    int group = (int)std::max<size_t>(1, std::min<size_t>(ns, kRefineBytes / h32));
     CgFields work{};
     void *rb, *eb;
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 121, h32 * group, &rb));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 120, h32 * group, &eb));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 115, h32 * group, &work.r));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 116, h32 * group, &work.p));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 117, h32 * group, &work.w));
-    QXD_TRY(qxd_ws(ctx, WS_SOLVER + 118, h32 * group, &work.t));
+    for (;; group = (group + 1) / 2) {  // fewer at a time where there is no memory for them
+        const std::pair<int, void**> fields[] = {{121, &rb}, {120, &eb}, {115, &work.r}, {116, &work.p}, {117, &work.w}, {118, &work.t}};
+        int rc = QXD_OK;
+        for (const auto& f : fields)
+            if (rc == QXD_OK) rc = qxd_ws(ctx, WS_SOLVER + f.first, h32 * group, f.second);
+        if (rc == QXD_OK) break;
+        if (group == 1) return rc;
+        for (const auto& f : fields) qxd_ws_free(ctx, WS_SOLVER + f.first);
+    }
     double worst = 0.0;
     for (int j0 = 0; j0 < ns; j0 += group) {
         std::vector<int> open;  // shifts of the group that miss the tolerance
