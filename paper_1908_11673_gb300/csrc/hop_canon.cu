@@ -15,8 +15,8 @@
 // Why: the conversion passes move four spinors per site and right-hand side (384 bytes in
 // FP32, more than the operator itself with many right-hand sides) and cost two to four
 // launches.  Time per call, conversion passes -> here (FP32 unless said): Dhat 8^4 24.6 ->
-// 16.1 us, Dhat^+ 24^3x48 147 -> 126 us, Dhat 32^3x64 C* 771 -> 685 us, D_w 24^3x48 with 12
-// right-hand sides 1521 -> 1102 us, D_w 24^3x48 FP64 1677 -> 1336 us (FP64-pipe bound: one
+// 6.1 us, Dhat^+ 24^3x48 146 -> 105 us, Dhat 32^3x64 C* 771 -> 585 us, D_w 24^3x48 with 12
+// right-hand sides 1500 -> 762 us, D_w 24^3x48 FP64 1674 -> 1331 us (FP64-pipe bound: one
 // launch over both parities also ends in one tail instead of two).
 #include <cstdio>
 
@@ -72,8 +72,13 @@ __device__ __forceinline__ void st32(double* p, const double v[4]) {
                  : "memory");
 }
 
-// bfloat16 storage: the values that a field of that precision would hold
-__device__ __forceinline__ float round_bf16(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+// bfloat16 storage: the values that a field of that precision would hold.  Two at a time: half the
+// conversions (with one at a time and no register bound, below, Dhat on 32^3x64 C* took 741 us).
+__device__ __forceinline__ cplx<float> round_bf16(float re, float im) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(re, im);
+    const unsigned u = *reinterpret_cast<const unsigned*>(&v);
+    return {__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)};
+}
 
 template <int P, bool RW>
 __device__ __forceinline__ void load_canon(const void* base, long long site, cplx<typename Prec<P>::real> s[12]) {
@@ -88,7 +93,7 @@ __device__ __forceinline__ void load_canon(const void* base, long long site, cpl
     }
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-        if constexpr (P == 2) s[k] = {round_bf16(v[2 * k]), round_bf16(v[2 * k + 1])};
+        if constexpr (P == 2) s[k] = round_bf16(v[2 * k], v[2 * k + 1]);
         else s[k] = {v[2 * k], v[2 * k + 1]};
     }
 }
@@ -101,8 +106,10 @@ __device__ __forceinline__ void store_canon(void* base, long long site, const cp
     R v[24];
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-        v[2 * k] = P == 2 ? (R)round_bf16((float)s[k].re) : s[k].re;
-        v[2 * k + 1] = P == 2 ? (R)round_bf16((float)s[k].im) : s[k].im;
+        cplx<R> c = s[k];
+        if constexpr (P == 2) c = round_bf16(c.re, c.im);
+        v[2 * k] = c.re;
+        v[2 * k + 1] = c.im;
     }
 #pragma unroll
     for (int k = 0; k < NL; ++k) st32(p + NV * k, v + NV * k);
@@ -154,10 +161,14 @@ __device__ __forceinline__ void canon_hop(const Geo& g, const CanonDev& a, const
 // 104, Dhat 32^3x64 C* 685 -> 585 (1952 bytes per even site at 7.0 TB/s).  With many
 // right-hand sides the L1 data pipe is 76 % busy: a 96-byte stride takes two passes per
 // 256-bit load where the internal layout takes one.
+// With bfloat16 storage the rounding makes the compiler take up to 228 registers (8 warps per
+// SM), so there the bound is 16 blocks (128 registers): Dhat 32^3x64 C* 645 us with 12 blocks,
+// 593 with 16, 620 with 20, and 671 by the conversion passes; four right-hand sides 2006, 1708,
+// 1796 and 2063.
 constexpr int kCanonThreads = 32;
 
 template <int P, int MODE>
-__global__ void __launch_bounds__(256, 1) k_hop_canon(Geo g, CanonDev a, int nrhs, int first, int end) {
+__global__ void __launch_bounds__(P == 2 ? 32 : 256, P == 2 ? 16 : 1) k_hop_canon(Geo g, CanonDev a, int nrhs, int first, int end) {
     using R = typename Prec<P>::real;
     const int rhs = blockIdx.x % nrhs;
     const int i = first + (blockIdx.x / nrhs) * kCanonThreads + threadIdx.x;
