@@ -98,9 +98,9 @@ __device__ __forceinline__ void vlink_for(const Geo& g, const PtcLinks& L, int d
         for (int j = 0; j < 3; ++j) V.a[i][j] = lk.z * lk.m.a[i][j];
 }
 
-// t = V s (forwards) or V^+ s on the colours of a spinor.  Scalar FP32 instructions run at
-// half the rate of the packed ones on this GPU (39 against 67 TFLOP/s measured): a packed
-// multiply-add takes the real or the imaginary part of an entry times a complex number.
+// t = V s (forwards) or V^+ s on the colours of a spinor.  Chains of multiply-adds with three
+// register operands reach 39 TFLOP/s as scalar instructions and 67 as packed ones (measured): a
+// packed multiply-add takes the real or the imaginary part of an entry times a complex number.
 __device__ __forceinline__ void transport_v(const Mat3<float>& V, bool fwd, const cplx<float> s[12],
                                             cplx<float> t[12]) {
 #pragma unroll
@@ -133,35 +133,36 @@ struct PtcParity {
 
 // ---- forward layer ------------------------------------------------------------------
 // Per colour a layer is the complex product of the (c, s) x (d, c', s') weights with the
-// transports.  A CTA takes 64 sites of one parity and goes over the 9 cin pairs (d, c') eight
+// transports.  A CTA takes 32 sites of one parity and goes over the 9 cin pairs (d, c') eight
 // at a time: its threads form the transports of eight pairs (a thread one site and two
 // pairs) in shared memory, then every thread multiplies: one site, all colours, NC output
-// channels, the eight warps split over two site groups, CG channel groups and KG groups of
-// the pairs (whose sums are added at the end, in a fixed order).
+// channels, the four warps split over CG channel groups and KG groups of the pairs (whose
+// sums are added at the end, in a fixed order).
 //
-// Bound by the FP32 pipe: 27,648 complex multiply-adds per site for 8 -> 8 channels, 194 us
-// on 16^4.  Two spin rows share a packed FP32 instruction; weights are read as broadcasts
-// of whole rows (real, imaginary and negated imaginary planes, so that no sign is formed in
-// the loop), each transport is loaded once per 8 rows.  One thread per (site, colour row)
-// with scalar arithmetic (every transport formed three times, weights re-read per row) took
-// 647 us for 8 -> 8 channels on 16^4; here 424 us (39 us for
-// 1 -> 8 channels, 86 us for 8 -> 1 with even outputs only; 133 us both before). 46 % of the
-// issue slots: what is left besides the products is the staging of the transports, which the
-// two resident CTAs overlap only in part.
-constexpr int kPtcSites = 64;
-constexpr int kPtcThreads = 256;
+// FP32 pipe: 27,648 complex multiply-adds per site for 8 -> 8 channels, 194 us on 16^4.  Two
+// spin rows share a packed FP32 instruction; weights are read as broadcasts of whole rows
+// (real and imaginary planes), each transport is loaded once per 8 rows.  What is left besides
+// the products is the staging of the transports, which the resident CTAs overlap only in
+// part.  8 -> 8 channels on 16^4: 647 us with one thread per (site, colour row) and scalar
+// arithmetic (every transport formed three times), 333 us here; 36 us for 1 -> 8, 86 us for
+// 8 -> 1 with even outputs only (133 us both before).  Three CTAs of four warps per SM with
+// 168 registers: the 70 layers of ten training pairs took 16.3 ms with two CTAs of eight
+// warps and 128 registers (spills) and a third weight plane, 14.9 ms so, 15.6 ms with four
+// CTAs, 15.9 ms with 16 rows per thread.
+constexpr int kPtcSites = 32;
+constexpr int kPtcThreads = 128;
 constexpr int kPtcPairs = 8;   // (d, c') pairs of a stage
 constexpr int kPtcGroup = 8;   // output channels per block (grid.z splits larger layers)
 
 struct PtcFwdShared {
     float2 t[4 * kPtcPairs][3][kPtcSites];
-    float w[3][4 * kPtcPairs][4 * kPtcGroup];  // Re W, Im W, -Im W
+    float w[2][4 * kPtcPairs][4 * kPtcGroup];  // Re W, Im W
 };
 
 // weight planes of a layer cin -> cout (adjoint: of the adjoint of the layer cout -> cin with
 // the weights W, W'[c][c'][d] = W[c'][c][opposite(d)]^+): [group of 8 output channels]
 // [pair q = d cin + c'][Re, Im, -Im][s'][4 (c - c0) + s], zero beyond cout
-constexpr int kPlane = 3 * 4 * 4 * kPtcGroup;  // floats of a pair
+constexpr int kPlane = 2 * 4 * 4 * kPtcGroup;  // floats of a pair
 
 __global__ void k_ptc_planes(const float2* __restrict__ W, int cin, int cout, int adjoint, float* __restrict__ P) {
     const int np = 9 * cin, n = ((cout + kPtcGroup - 1) / kPtcGroup) * np * 4 * 4 * kPtcGroup;
@@ -179,23 +180,22 @@ __global__ void k_ptc_planes(const float2* __restrict__ W, int cin, int cout, in
         float* o = P + ((size_t)z * np + q) * kPlane + si * 4 * kPtcGroup + row;
         o[0] = v.x;
         o[16 * kPtcGroup] = v.y;
-        o[32 * kPtcGroup] = -v.y;
     }
 }
 
 template <int NC, int CG, int KG>
-__global__ void __launch_bounds__(kPtcThreads, 2) k_ptc_fwd(Geo g, PtcLinks L, const float4* __restrict__ a, int cin,
+__global__ void __launch_bounds__(kPtcThreads, 3) k_ptc_fwd(Geo g, PtcLinks L, const float4* __restrict__ a, int cin,
                                                            int cout, const float* __restrict__ planes,
                                                            float4* __restrict__ out, PtcParity par) {
-    static_assert(CG * KG == 4, "eight warps: two site groups, CG channel and KG pair groups");
+    static_assert(CG * KG == 4, "four warps: CG channel and KG pair groups");
     extern __shared__ float4 ptc_sh[];
     PtcFwdShared& S = *reinterpret_cast<PtcFwdShared*>(ptc_sh);
     constexpr int R = 4 * NC;       // rows of a thread
     const int c0 = blockIdx.z * kPtcGroup;
     const int ng = min(kPtcGroup, cout - c0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int sg = warp & 1, cg = (warp >> 1) % CG, kg = (warp >> 1) / CG;
-    const int site = 32 * sg + lane;
+    const int cg = warp % CG, kg = warp / CG;
+    const int site = lane;
     const int st_site = tid & (kPtcSites - 1), st_slot = tid / kPtcSites;
     const size_t chs = (size_t)12 * g.Vh;  // float4 per channel
     const int tiles = (g.Vh + kPtcSites - 1) / kPtcSites;
@@ -251,9 +251,9 @@ __global__ void __launch_bounds__(kPtcThreads, 2) k_ptc_fwd(Geo g, PtcLinks L, c
             for (int kk = 0; kk < 4 * kPtcPairs / KG; ++kk) {
                 const int k = kg * (4 * kPtcPairs / KG) + kk;
                 if (k >= 4 * np) break;
-                float2 w[3][R / 2];
+                float2 w[2][R / 2];
 #pragma unroll
-                for (int f = 0; f < 3; ++f)
+                for (int f = 0; f < 2; ++f)
 #pragma unroll
                     for (int r = 0; r < R / 4; ++r) {
                         const float4 v = *reinterpret_cast<const float4*>(&S.w[f][k][R * cg + 4 * r]);
@@ -263,10 +263,10 @@ __global__ void __launch_bounds__(kPtcThreads, 2) k_ptc_fwd(Geo g, PtcLinks L, c
 #pragma unroll
                 for (int i = 0; i < 3; ++i) {
                     const float2 t = S.t[k][i][site];
-                    const float2 tr = make_float2(t.x, t.x), ti = make_float2(t.y, t.y);
+                    const float2 tr = make_float2(t.x, t.x), ti = make_float2(t.y, t.y), tn = make_float2(-t.y, -t.y);
 #pragma unroll
                     for (int r = 0; r < R / 2; ++r) {
-                        re[r][i] = fma2(w[2][r], ti, fma2(w[0][r], tr, re[r][i]));
+                        re[r][i] = fma2(w[1][r], tn, fma2(w[0][r], tr, re[r][i]));
                         im[r][i] = fma2(w[1][r], tr, fma2(w[0][r], ti, im[r][i]));
                     }
                 }
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kPtcThreads, 2) k_ptc_fwd(Geo g, PtcLinks L, c
             constexpr int NV = 3 * R;  // float2 values of a thread
             __syncthreads();
             if (kg > 0) {
-                float2* o = red + (size_t)(((kg - 1) * CG + cg) * 2 + sg) * NV * 32 + lane;
+                float2* o = red + (size_t)((kg - 1) * CG + cg) * NV * 32 + lane;
 #pragma unroll
                 for (int r = 0; r < R / 2; ++r)
 #pragma unroll
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kPtcThreads, 2) k_ptc_fwd(Geo g, PtcLinks L, c
             __syncthreads();
             if (kg == 0) {
                 for (int k = 1; k < KG; ++k) {
-                    const float2* o = red + (size_t)(((k - 1) * CG + cg) * 2 + sg) * NV * 32 + lane;
+                    const float2* o = red + (size_t)((k - 1) * CG + cg) * NV * 32 + lane;
 #pragma unroll
                     for (int r = 0; r < R / 2; ++r)
 #pragma unroll
@@ -878,7 +878,7 @@ static size_t plane_floats(int cin, int cout) {
     return (size_t)((cout + kPtcGroup - 1) / kPtcGroup) * 9 * cin * kPlane;
 }
 static int launch_planes(qxd_ctx* ctx, const float2* W, int cin, int cout, bool adjoint, float* P, cudaStream_t st) {
-    const long long n = (long long)plane_floats(cin, cout) / 3;
+    const long long n = (long long)plane_floats(cin, cout) / 2;
     k_ptc_planes<<<nblocks(n, 256), 256, 0, st>>>(W, cin, cout, adjoint ? 1 : 0, P);
     QXD_CUDA(ctx, cudaGetLastError());
     return QXD_OK;

@@ -27,7 +27,7 @@
 // Bound by latency and shared-memory loads (35 % of the issue slots, 49 % of the LSU; the
 // site-diagonal terms of each step come from L2).  Per lane and direction a colour product is
 // 18 packed multiply-adds, (Re, Im) of a link entry times a duplicated part of the
-// half-spinor; scalar FP32 runs at half the packed rate.  Directions are unrolled with the
+// half-spinor (half the instructions).  Directions are unrolled with the
 // half's signs as factors: a run-time loop with selects took 2.6 times the instructions.
 // Sweep of 24^3x48 with nmr = 5: 499 us so, 496 us with few instructions but strided reads
 // and bank conflicts, 276 us with the blocks' own copies and spins interleaved.
