@@ -162,7 +162,9 @@ void qxd_destroy(qxd_ctx* ctx);
  * constraint U(x + L1 e1) = U(x)^*, A(x + L1 e1) = -A(x) (eq. cstar-bc-gauge).
  * invqel = 1/qel (elementary charge) is kept for reference; the operator does not
  * depend on it (q Ahat = qhat (i/4) Im sum z_{mu nu}).
- * Invalidates every SW term set before.  Synchronises `stream`. */
+ * Invalidates every SW term set before; their device memory is kept for the next
+ * qxd_set_clover of the same slots (and given back when the context runs short of
+ * memory).  Synchronises `stream`. */
 int qxd_set_links(qxd_ctx* ctx, const double* U, const double* A, double invqel, void* stream);
 
 /* Build, for flavour slot fl (0..7), the hopping phases z^qhat (with the
@@ -280,10 +282,11 @@ int qxd_sdet(qxd_ctx* ctx, int fl, double* logdet, int* nneg, void* stream);
  *    and arrays on another GPU return QXD_EARG (staging would allocate).
  *  - The first call on a device looks up the array's device address with the
  *    CUDA runtime.  Make that first call before any stream capture.
- *  - The call never runs the launch-shape autotuner of qxd_apply_Dhat_eo (which
- *    times candidate shapes and waits for them on the host): it uses the shape
- *    that an earlier qxd_apply_Dhat_eo on the same context and lattice tuned,
- *    else a fixed default shape.  The result is the same either way.
+ *  - The call never runs the launch-shape autotuner (which times candidate shapes
+ *    and waits for them on the host).  Fields that are not 32-byte aligned, or that
+ *    overlap in part, take kernels that it tunes: there the call uses the shape that
+ *    an earlier qxd_apply_Dhat_eo of such fields on the same context and lattice
+ *    tuned, else a fixed default shape.  The result is the same either way.
  *  - Every call, from any context on the device, uses the same array.  Calls
  *    whose work overlaps on the GPU (different streams, or different threads)
  *    race and give wrong results.  Serialise them.  Each call overwrites the
@@ -311,7 +314,9 @@ int qxd_set_precond_weights(qxd_ctx* ctx, int fl, const float* W, int nlayers, i
  * (hops leaving the block dropped) approximately by nmr minimal-residual steps on
  * the block's even-odd system, for the residual rho = eta - D psi taken on the
  * block at the start of its colour's sweep.  FGCR on Dhat uses z_e = (M (r_e, 0))_e (Dhat^-1 = (D^-1)_ee).
- * Arithmetic in FP32. */
+ * Arithmetic in FP32.  The first sweep after qxd_set_clover lays the links and
+ * site-diagonal terms out by block (720 bytes of device memory per site and flavour
+ * slot, given back when the context runs short of memory; not under stream capture). */
 
 /* Set ncy and nmr (1..64 each; default 5 and 5, the paper's values). */
 int qxd_set_sap(qxd_ctx* ctx, int ncy, int nmr);

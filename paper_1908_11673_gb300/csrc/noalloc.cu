@@ -91,6 +91,9 @@ extern "C" int qxd_apply_Dhat_eo_noalloc(qxd_ctx* ctx, int fl, int prec, int dag
     void* oe = scratch + 2 * kNoallocFieldBytes;
     cudaStream_t st = (cudaStream_t)stream;
     const int cprec = prec == QXD_FP64 ? 0 : 1;
+    // on the caller's fields as qxd_apply_Dhat_eo does it (8^4 FP32: 24 -> 6 us)
+    if (canon_fits(in_e, out_e, (size_t)ctx->g.Vh * 12 * (cprec == 0 ? 16 : 8), true))
+        return op_Dhat_canon(ctx, fl, prec, dagger ? 1 : 0, in_e, out_e, to, 1, st);
     NoAutotune frozen;
     QXD_TRY(launch_pack(ctx, cprec, in_e, 0, 0, prec, ie, 1, st));
     QXD_TRY(op_Dhat(ctx, fl, prec, dagger ? 1 : 0, ie, oe, to, st, 1));
