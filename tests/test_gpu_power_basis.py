@@ -1,11 +1,12 @@
 """Unpreconditioned FP32 inner solves from the shifted power basis.
 
 Restart lengths on both sides of where the inner products split (8) and of where the
-power basis ends (16), one step per cycle, a budget that ends within a cycle, and an
+power basis ends (16), one step per cycle, a budget that ends within a cycle, an
 operator proportional to the identity up to the site-diagonal term (a basis that is used
-up after a few steps), a residual almost in the operator's kernel.  Solutions are held to the requested true residual with the FP64
-oracle; the iteration count of a restart length is that of GCR, whose iterates the method
-reproduces in exact arithmetic, to within one cycle per outer step.
+up after a few steps), and a residual almost in the operator's kernel.  Solutions are held
+to the requested true residual with the FP64 oracle; the iteration count of a restart
+length is that of GCR, whose iterates the method reproduces in exact arithmetic, to within
+one cycle per outer step.
 """
 import numpy as np
 import pytest
