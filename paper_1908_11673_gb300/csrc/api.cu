@@ -288,6 +288,13 @@ int qxd_set_links(qxd_ctx* ctx, const double* U, const double* A, double invqel,
     const void *dU, *dA;
     QXD_TRY(stage_in(ctx, WS_STAGE_U, U, Vp * 4 * 9 * 16, &dU, st));
     QXD_TRY(stage_in(ctx, WS_STAGE_A, A, Vp * 4 * 8, &dA, st));
+    // operators may still run on other streams with the links that are overwritten here (and
+    // with the flavours' fields, which are kept and which qxd_set_clover overwrites)
+    for (const auto& F : ctx->fl)
+        if (F.V64) {
+            QXD_CUDA(ctx, cudaDeviceSynchronize());
+            break;
+        }
     for (auto& F : ctx->fl) reset_flavour(F);
     QXD_TRY(launch_set_links(ctx, static_cast<const double2*>(dU), static_cast<const double*>(dA), st));
     QXD_CUDA(ctx, cudaStreamSynchronize(st));
