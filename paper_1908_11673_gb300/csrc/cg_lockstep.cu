@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_direction(int Vh, CgDev c, in
 }  // namespace
 
 int cg_lockstep(qxd_ctx* ctx, int fl, int B, bool normal, const double* sigma, const double* rtol, const void* bv,
-                void* ev, const CgFields& work, long long budget, int* iters, cudaStream_t st) {
+                void* ev, const CgFields& work, long long budget, int each, int* iters, cudaStream_t st) {
     if (B < 1 || B > kCgMax) return qxd_fail(ctx, QXD_EARG, "lockstep CG: 1 to 32 right-hand sides");
     const Geo& g = ctx->g;
     const QxdFlavour& F = ctx->fl[fl];
@@ -446,14 +446,14 @@ int cg_lockstep(qxd_ctx* ctx, int fl, int B, bool normal, const double* sigma, c
         return QXD_OK;
     };
     int chunk = 0, looked = 0;  // chunks launched and looked at
-    while (rc == QXD_OK && running > 0) {
+    while (rc == QXD_OK && running > 0 && it < each) {  // what still runs has made `it` iterations
         long long left = budget - total - (long long)(it - seen) * running;
         if (left <= 0 && looked < chunk) {  // count what was really made
             rc = look(looked++ & 1);
             continue;
         }
         if (left <= 0) break;
-        const int n = (int)std::max<long long>(1, std::min<long long>(kChunk, left / running));
+        const int n = (int)std::max<long long>(1, std::min<long long>({kChunk, left / running, each - it}));
         for (int k = 0; k < n; ++k) iteration(it++);
         const int turn = chunk++ & 1;
         launched[turn] = it;

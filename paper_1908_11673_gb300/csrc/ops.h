@@ -71,13 +71,13 @@ void dfl_free(QxdFlavour& F);
 // Conjugate gradients of B <= 32 FP32 right-hand sides in lockstep (cg_lockstep.cu), fields
 // one after the other: normal = false solves (Dhat^+ Dhat + sigma[j]) e_j = b_j, true
 // min |b_j - Dhat e_j| on the normal equations; right-hand side j stops at rtol[j] |b_j|
-// (rtol >= 1: e_j = 0), all of them once `budget` iterations were made together; iters[j]
-// receives its iterations.  work: B fields each (z only with normal).
+// (rtol >= 1: e_j = 0) or after `each` iterations, all of them once `budget` iterations were
+// made together; iters[j] receives its iterations.  work: B fields each (z only with normal).
 struct CgFields {
     void *r, *z, *p, *w, *t;
 };
 int cg_lockstep(qxd_ctx* ctx, int fl, int B, bool normal, const double* sigma, const double* rtol, const void* b,
-                void* e, const CgFields& work, long long budget, int* iters, cudaStream_t st);
+                void* e, const CgFields& work, long long budget, int each, int* iters, cudaStream_t st);
 
 // solvers.cu
 int solve_cgne64(qxd_ctx* ctx, int fl, const qxd_solver* s, const Full& eta, const Full& x, qxd_info* info,

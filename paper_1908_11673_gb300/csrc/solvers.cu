@@ -157,7 +157,8 @@ int cgnr_inner(qxd_ctx* ctx, int fl, int P, const void* b, void* e, int max_iter
     QXD_TRY(qxd_ws(ctx, WS_SOLVER + 103, hb, &w));
     QXD_TRY(qxd_ws(ctx, WS_SOLVER + 104, hb, &to));
     if (P == QXD_FP32)
-        return cg_lockstep(ctx, fl, 1, true, nullptr, &rtol, b, e, CgFields{sv, z, p, w, to}, max_iter, iters, st);
+        return cg_lockstep(ctx, fl, 1, true, nullptr, &rtol, b, e, CgFields{sv, z, p, w, to}, max_iter, max_iter, iters,
+                           st);
     QXD_CUDA(ctx, cudaMemsetAsync(e, 0, hb, st));
     QXD_CUDA(ctx, cudaMemcpyAsync(sv, b, hb, cudaMemcpyDeviceToDevice, st));
     QXD_TRY(op_Dhat(ctx, fl, P, 1, sv, z, to, st));
@@ -1080,7 +1081,7 @@ int solve_mscg(qxd_ctx* ctx, int fl, int ns, const double* sigma, const qxd_solv
             if (open.empty()) break;
             std::vector<int> its(open.size(), 0);
             QXD_TRY(cg_lockstep(ctx, fl, (int)open.size(), false, sig.data(), rtol.data(), rb, eb, work,
-                                s->nmx - info->iters, its.data(), st));
+                                s->nmx - info->iters, s->nmx - info->iters, its.data(), st));
             for (size_t i = 0; i < open.size(); ++i) {
                 info->iters += its[i];
                 QXD_TRY(blas_axpby(ctx, 1, 0, n, 1.0, 0.0, static_cast<char*>(eb) + i * h32, 1.0, 0.0,
@@ -1482,9 +1483,9 @@ int solve_fgcr_dc_batched(qxd_ctx* ctx, int fl, const qxd_solver* s, const Full&
             const CgFields work{ra, za, at(za, hbP, G), wa, at(wa, hbP, G)};
             for (int j = 0; j < B; j += G) {
                 const int nb = std::min(G, B - j);
-                const long long each = s->nmx - info->iters;
-                QXD_TRY(cg_lockstep(ctx, fl, nb, true, nullptr, &ctol[j], at(bP, hbP, j), at(eeP, hbP, j), work, each * nb,
-                                    &it[j], st));
+                const int each = s->nmx - info->iters;
+                QXD_TRY(cg_lockstep(ctx, fl, nb, true, nullptr, &ctol[j], at(bP, hbP, j), at(eeP, hbP, j), work,
+                                    (long long)each * nb, each, &it[j], st));
             }
             for (int j = 0; j < B; ++j) mx = std::max(mx, 2 * it[j]);
         } else if (use_cgnr) {
