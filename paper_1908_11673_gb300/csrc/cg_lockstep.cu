@@ -430,6 +430,8 @@ int cg_lockstep(qxd_ctx* ctx, int fl, int B, bool normal, const double* sigma, c
     int it = 0, seen = 0, launched[2] = {0, 0};
     long long total = 0;
     std::vector<int> done(B, 0);
+    std::vector<char> runs(B);
+    for (int j = 0; j < B; ++j) runs[j] = rtol[j] < 1.0;
     auto look = [&](int turn) -> int {
         if (cudaEventSynchronize(ev2[turn]) != cudaSuccess) return qxd_fail(ctx, QXD_ECUDA, "lockstep CG: wait failed");
         seen = launched[turn];
@@ -439,20 +441,30 @@ int cg_lockstep(qxd_ctx* ctx, int fl, int B, bool normal, const double* sigma, c
             const int cv = flags[turn][j], bad = flags[turn][kCgMax + j];
             if (bad == 1) return qxd_fail(ctx, QXD_ENAN, "non-finite value in CG");
             if (bad == 2) return qxd_fail(ctx, QXD_EBREAKDOWN, "shifted CG: <p, A p> <= 0");
-            done[j] = cv == INT_MAX ? seen : cv + 1;
+            runs[j] = cv == INT_MAX;
+            done[j] = runs[j] ? seen : cv + 1;
             total += done[j];
-            running += cv == INT_MAX;
+            running += runs[j];
         }
         return QXD_OK;
     };
     int chunk = 0, looked = 0;  // chunks launched and looked at
     while (rc == QXD_OK && running > 0 && it < each) {  // what still runs has made `it` iterations
         long long left = budget - total - (long long)(it - seen) * running;
-        if (left <= 0 && looked < chunk) {  // count what was really made
+        if (left < running && looked < chunk) {  // count what was really made
             rc = look(looked++ & 1);
             continue;
         }
         if (left <= 0) break;
+        const int stop = it - 1;
+        for (int j = B - 1; j >= 0 && left < running; --j) {  // not one more iteration for all of them
+            if (!runs[j]) continue;
+            runs[j] = 0;
+            running -= 1;
+            if (cudaMemcpyAsync(c.s->conv + j, &stop, sizeof stop, cudaMemcpyHostToDevice, st) != cudaSuccess)
+                rc = qxd_fail(ctx, QXD_ECUDA, "lockstep CG: copy failed");
+        }
+        if (rc != QXD_OK) break;
         const int n = (int)std::max<long long>(1, std::min<long long>({kChunk, left / running, each - it}));
         for (int k = 0; k < n; ++k) iteration(it++);
         const int turn = chunk++ & 1;

@@ -22,3 +22,17 @@ def test_right_hand_sides_that_stop_leave_nothing_to_the_others(nrhs, nmx):
     info = ctx.solve(0, eta, psi, nkv=2, inner=qxd.FP32, nrhs=nrhs, tol=1e-10, nmx=nmx, check=False)
     assert info.status == 2 and nmx <= info.iters <= 2 * nmx
     ctx.close()
+
+
+def test_shifts_share_exactly_what_is_left():
+    qxd, ctx, op, _, _ = setup((4, 4, 6, 6), 1, PI, qhat=4, kappa=0.13)
+    phi = workload.spinor(op.geom.V // 2, 5)
+    sigma = [0.0, 1e-3, 8.4, 1e-6, 500.0, 0.3]
+    x = np.empty((len(sigma),) + phi.shape, dtype=np.complex128)
+    full = ctx.solve_multishift(0, sigma, phi, x, tol=1e-11, inner=qxd.FP32).iters
+    for nmx in range(full // 3, full, 3):  # some of these end in the middle of a step of all shifts
+        info = ctx.solve_multishift(0, sigma, phi, x, tol=1e-11, inner=qxd.FP32, nmx=nmx, check=False)
+        assert info.status == 2 and info.iters <= nmx, nmx
+    again = ctx.solve_multishift(0, sigma, phi, x, tol=1e-11, inner=qxd.FP32, nmx=full)
+    assert again.iters == full
+    ctx.close()
