@@ -1,7 +1,7 @@
 // Second half of Dhat with the inner products of a GCR step fused into its epilogue
 // (Sec. 2.3 operator; the solver of Sec. 4.4).
 //
-//   w = A_ee r - H_eo t - shift r,   t = A_oo^-1 H_oe r  (the first half, an ordinary launch)
+//   w = scale (A_ee r - H_eo t - shift r),   t = A_oo^-1 H_oe r  (the first half, an ordinary launch)
 //
 // The solver that applies Dhat to its direction r (the current residual of GCR, or the last
 // vector of a shifted power basis) next needs <W_j, w> for the K earlier basis fields,
@@ -40,7 +40,8 @@ constexpr int kDotsFlush = 8;
 
 // T threads per block: 64 where blocks of 256 would leave most of the chip without one
 template <int K, int T>
-__global__ void __launch_bounds__(T, 512 / T) k_hop_dots(Geo g, HopDev a, float shift, MultiPtr W, RedOut o) {
+__global__ void __launch_bounds__(T, 512 / T) k_hop_dots(Geo g, HopDev a, float shift, float scale, MultiPtr W,
+                                                        RedOut o) {
     constexpr int NC = 2 * K + 4;
     __shared__ double vs[NC][T];
     float fa[NC];
@@ -81,6 +82,8 @@ __global__ void __launch_bounds__(T, 512 / T) k_hop_dots(Geo g, HopDev a, float 
 #pragma unroll
                 for (int k = 0; k < 12; ++k) acc[k] = {fmaf(-shift, r[k].re, acc[k].re), fmaf(-shift, r[k].im, acc[k].im)};
             }
+#pragma unroll
+            for (int k = 0; k < 12; ++k) acc[k] = scale * acc[k];
             dot_site(r, acc, fa[2 * K], fa[2 * K + 1]);
         }
         store_spinor<1>(out, g.Vh, h, acc);
@@ -150,18 +153,18 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_hop_resid(Geo g, HopDev a, c
 }
 
 template <int K, int T>
-void launch_kt(qxd_ctx* ctx, const HopDev& d, float shift, const MultiPtr& W, int slot, cudaStream_t st) {
+void launch_kt(qxd_ctx* ctx, const HopDev& d, float shift, float scale, const MultiPtr& W, int slot, cudaStream_t st) {
     int nb = wave_blocks(ctx, k_hop_dots<K, T>, T, (size_t)T, (size_t)ctx->g.Vh);
     const int cap = kPartials / (2 * K + 4);  // partial sums of every block fit the buffer
     if (nb > cap) nb = cap;
-    k_hop_dots<K, T><<<nb, T, 0, st>>>(ctx->g, d, shift, W, red_out(ctx, slot));
+    k_hop_dots<K, T><<<nb, T, 0, st>>>(ctx->g, d, shift, scale, W, red_out(ctx, slot));
 }
 
 template <int K>
-void launch_k(qxd_ctx* ctx, const HopDev& d, float shift, const MultiPtr& W, int slot, cudaStream_t st) {
+void launch_k(qxd_ctx* ctx, const HopDev& d, float shift, float scale, const MultiPtr& W, int slot, cudaStream_t st) {
     // less than one wave of 256-thread blocks (two per SM)
-    if (ctx->g.Vh < 512 * ctx->nsm) launch_kt<K, 64>(ctx, d, shift, W, slot, st);
-    else launch_kt<K, kRedThreads>(ctx, d, shift, W, slot, st);
+    if (ctx->g.Vh < 512 * ctx->nsm) launch_kt<K, 64>(ctx, d, shift, scale, W, slot, st);
+    else launch_kt<K, kRedThreads>(ctx, d, shift, scale, W, slot, st);
 }
 
 }  // namespace
@@ -195,8 +198,8 @@ int launch_hop_resid(qxd_ctx* ctx, int fl, const HopArgs& a, const void* b, int 
     return QXD_OK;
 }
 
-int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* const* W, double shift, int slot,
-                    cudaStream_t st) {
+int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* const* W, double shift, double scale,
+                    int slot, cudaStream_t st) {
     if (k < 0 || k > kMultiMax) return qxd_fail(ctx, QXD_EARG, "fused hop: at most 8 basis fields");
     if (a.self_mode != 1 || a.post_mode != 0 || a.nrhs != 1 || a.g5_nb || a.g5_self || a.g5_out)
         return qxd_fail(ctx, QXD_EARG, "fused hop: only the second half of Dhat, one right-hand side");
@@ -208,15 +211,15 @@ int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* c
     // neighbours + self + output 3 x 96) and the K basis fields
     ProfScope prof(ctx, "hop_fp32_self1_post0_dots", (double)Vh * (8 * 56.0 + 288.0 + 96.0 * (3 + k)), st);
     switch (k) {
-        case 0: launch_k<0>(ctx, d, (float)shift, mp, slot, st); break;
-        case 1: launch_k<1>(ctx, d, (float)shift, mp, slot, st); break;
-        case 2: launch_k<2>(ctx, d, (float)shift, mp, slot, st); break;
-        case 3: launch_k<3>(ctx, d, (float)shift, mp, slot, st); break;
-        case 4: launch_k<4>(ctx, d, (float)shift, mp, slot, st); break;
-        case 5: launch_k<5>(ctx, d, (float)shift, mp, slot, st); break;
-        case 6: launch_k<6>(ctx, d, (float)shift, mp, slot, st); break;
-        case 7: launch_k<7>(ctx, d, (float)shift, mp, slot, st); break;
-        default: launch_k<8>(ctx, d, (float)shift, mp, slot, st); break;
+        case 0: launch_k<0>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
+        case 1: launch_k<1>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
+        case 2: launch_k<2>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
+        case 3: launch_k<3>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
+        case 4: launch_k<4>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
+        case 5: launch_k<5>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
+        case 6: launch_k<6>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
+        case 7: launch_k<7>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
+        default: launch_k<8>(ctx, d, (float)shift, (float)scale, mp, slot, st); break;
     }
     QXD_CUDA(ctx, cudaGetLastError());
     return QXD_OK;

@@ -83,10 +83,10 @@ static int dhat_first(qxd_ctx* ctx, int fl, const void* in_e, void* out_e, void*
 }
 
 int op_Dhat_dots(qxd_ctx* ctx, int fl, const void* in_e, void* out_e, void* tmp_o, int k, const void* const* W,
-                 double shift, int slot, cudaStream_t st) {
+                 double shift, double scale, int slot, cudaStream_t st) {
     HopArgs a;
     QXD_TRY(dhat_first(ctx, fl, in_e, out_e, tmp_o, &a, st));
-    return launch_hop_dots(ctx, fl, a, k, W, shift, slot, st);
+    return launch_hop_dots(ctx, fl, a, k, W, shift, scale, slot, st);
 }
 
 int op_Dhat_resid(qxd_ctx* ctx, int fl, const void* b_e, const void* e_e, void* r_e, void* tmp_o, int slot,

@@ -23,13 +23,13 @@ int op_Dw(qxd_ctx* ctx, int fl, int P, const Full& in, const Full& out, cudaStre
 int op_Dhat(qxd_ctx* ctx, int fl, int P, int dagger, const void* in_e, void* out_e, void* tmp_o, cudaStream_t st,
             int nrhs = 1);
 // Dhat on FP32 even fields (no dagger, one right-hand side) with the inner products of
-// a GCR step fused into the second half and out_e -= shift in_e: result[slot + 2j, +1] = <W_j, out_e> (j < k <= 8),
+// a GCR step fused into the second half and out_e = scale (Dhat in_e - shift in_e): result[slot + 2j, +1] = <W_j, out_e> (j < k <= 8),
 // [slot + 2k, +1] = <in_e, out_e>, [slot + 2k + 2] = |out_e|^2 over finite sites,
 // [slot + 2k + 3] = number of sites where it is not finite
 int op_Dhat_dots(qxd_ctx* ctx, int fl, const void* in_e, void* out_e, void* tmp_o, int k, const void* const* W,
-                 double shift, int slot, cudaStream_t st);
-int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* const* W, double shift, int slot,
-                    cudaStream_t st);
+                 double shift, double scale, int slot, cudaStream_t st);
+int launch_hop_dots(qxd_ctx* ctx, int fl, const HopArgs& a, int k, const void* const* W, double shift, double scale,
+                    int slot, cudaStream_t st);
 // r_e = b_e - Dhat e_e on FP32 even fields: result[slot] = |r|^2 over finite sites, [slot + 1]
 // the number of the others
 int op_Dhat_resid(qxd_ctx* ctx, int fl, const void* b_e, const void* e_e, void* r_e, void* tmp_o, int slot,

@@ -211,10 +211,12 @@ static int precond_into(qxd_ctx* ctx, int fl, int Pv, int Pb, int kind, const vo
 // Restarted minimal residuals without a preconditioner in FP32, restart lengths up to 16: in
 // exact arithmetic the iterates of GCR(nkv), from a basis that needs no vector update.
 //
-// A cycle forms z_0 = r, z_{k+1} = (Dhat - d) z_k with the inner products <z_j, z_{k+1}> from
+// A cycle forms z_0 = r, z_{k+1} = (Dhat - d) z_k / u_k with the inner products <z_j, z_{k+1}> from
 // the operator's second launch (from the ninth step on those with z_0 .. z_{k-9} in a pass of
-// their own), so that the Gram matrix G of z_0 .. z_K is known.  With
-// a_k = Dhat z_k = z_{k+1} + d_k z_k the correction sum_k c_k z_k of minimal residual solves
+// their own), so that the Gram matrix G of z_0 .. z_K is known.  The u_k are powers of two (exact)
+// that keep |z_k| near |r|: |Dhat - d| to the sixteenth power is 1e9 and more, and FP32 sums of
+// squares would overflow for sources of width 1e11.  With
+// a_k = Dhat z_k = u_k z_{k+1} + d_k z_k the correction sum_k c_k z_k of minimal residual solves
 // M c = <a, r>, M = (<a_i, a_k>), by a Cholesky factorisation that grows by one row per
 // step; its forward substitution gives the residual norm after every step.  d is the
 // Rayleigh quotient of the first residual: it centres the spectrum, so that the powers stay
@@ -262,23 +264,28 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
         }
     } ev{st};
     for (auto& x : ev.e) QXD_CUDA(ctx, cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
-    std::vector<double> d(nkv, 0.0);
+    const int m = nkv + 1;
+    std::vector<C> G(m * m), L(nkv * nkv), y(nkv), c(nkv);
+    std::vector<double> d(nkv, 0.0), u(nkv, 1.0);  // z_{k+1} = (Dhat - d_k) z_k / u_k
     double shift = 0.0;  // an FP32 number, as the kernel applies it
+    double growth = 0.0;  // log2 of |(Dhat - d) z_k| / |z_k|, the last one known
     bool centred = false;
-    auto launch = [&](int k) -> int {
+    // step k when the numbers of the steps before K are known
+    auto launch = [&](int k, int K) -> int {
         const int slot = k * k + 3 * k;
         d[k] = shift;
+        double size = 0.5 * std::log2(std::max(G[K * m + K].real() / G[0].real(), 1e-30)) + growth;  // of |z_{k+1}|
+        for (int i = K; i < k; ++i) size += growth - std::log2(u[i]);
+        u[k] = std::exp2(std::round(std::min(std::max(size, -60.0), 60.0)));
         const int rest = std::max(0, k - kMultiMax);
         QXD_TRY(op_Dhat_dots(ctx, fl, z[k], const_cast<void*>(z[k + 1]), to, k - rest, z.data() + rest, shift,
-                             slot + 2 * rest, st));
+                             1.0 / u[k], slot + 2 * rest, st));
         if (rest > 0) QXD_TRY(blas_multi_dot(ctx, QXD_FP32, n, rest, z.data(), z[k + 1], slot, st));
         QXD_CUDA(ctx, cudaMemcpyAsync(ctx->red_host + slot, ctx->red_result + slot, sizeof(double) * (2 * k + 4),
                                       cudaMemcpyDeviceToHost, st));
         QXD_CUDA(ctx, cudaEventRecord(ev.e[k & 1], st));
         return QXD_OK;
     };
-    const int m = nkv + 1;
-    std::vector<C> G(m * m), L(nkv * nkv), y(nkv), c(nkv);
     while (*iters < max_iter) {
         const double rr_cycle = rr;
         G[0] = rr;
@@ -286,10 +293,11 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
         int steps = std::min(nkv, max_iter - *iters), launched = 0, K = 0;
         bool reached = false, used_up = false;
         while (K < steps && !reached && !used_up) {
-            if (launched == K) QXD_TRY(launch(launched++));
+            if (launched == K) QXD_TRY(launch(launched++, K));
             // the next step is queued before this one's numbers are looked at, unless this one may
             // be the last
-            if (launched < steps && launched == K + 1 && centred && rr * drop > 4.0 * target) QXD_TRY(launch(launched++));
+            if (launched < steps && launched == K + 1 && centred && rr * drop > 4.0 * target)
+                QXD_TRY(launch(launched++, K));
             QXD_CUDA(ctx, cudaEventSynchronize(ev.e[K & 1]));
             const int k = K;
             const double* h = ctx->red_host + k * k + 3 * k;
@@ -300,17 +308,18 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
             }
             G[(k + 1) * m + k + 1] = h[2 * k + 2];
             // <z_i, a_k>, the new row of L and the new entry of y
-            auto za = [&](int i) { return G[i * m + k + 1] + d[k] * G[i * m + k]; };
+            auto za = [&](int i) { return u[k] * G[i * m + k + 1] + d[k] * G[i * m + k]; };
             double diag = 0.0;
             for (int i = 0; i <= k; ++i) {
-                C v = std::conj(za(i + 1) + d[i] * za(i));  // <a_k, a_i>
+                C v = std::conj(u[i] * za(i + 1) + d[i] * za(i));  // <a_k, a_i>
                 if (i == k) diag = v.real();
                 for (int q = 0; q < i; ++q) v -= L[k * nkv + q] * std::conj(L[i * nkv + q]);
                 L[k * nkv + i] = i < k ? v / L[i * nkv + i] : v;
             }
             // z_1 close to -d z_0 (a residual almost in the kernel): |Dhat z_0|^2 is lost in the
             // difference, from here on the powers are taken without a shift
-            const double scale = h[2 * k + 2] + d[k] * d[k] * G[k * m + k].real();
+            const double w2 = u[k] * u[k] * h[2 * k + 2];
+            const double scale = w2 + d[k] * d[k] * G[k * m + k].real();
             if (k == 0 && d[0] != 0.0 && !(diag > 1e-5 * scale)) {
                 shift = 0.0;
                 *iters += launched;
@@ -331,6 +340,7 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
             const double next = rr - std::norm(y[k]);
             drop = next > 0.0 ? next / rr : 0.0;
             rr = next;
+            if (w2 > 0.0) growth = 0.5 * std::log2(w2 / G[k * m + k].real());
             if (!centred) {
                 shift = (double)(float)(G[1].real() / G[0].real());
                 centred = true;
@@ -423,7 +433,7 @@ int fgcr_inner(qxd_ctx* ctx, int fl, int P, const qxd_solver* s, const void* b, 
             // own second launch (op_Dhat_dots), which also counts non-finite sites.
             double nonfinite = 0.0;
             if (rz && Pb == QXD_FP32 && k <= kMultiMax) {
-                QXD_TRY(op_Dhat_dots(ctx, fl, Z[k], W[k], to, k, W.data(), 0.0, 0, st));
+                QXD_TRY(op_Dhat_dots(ctx, fl, Z[k], W[k], to, k, W.data(), 0.0, 1.0, 0, st));
                 QXD_TRY(blas_fetch(ctx, 2 * k + 4, st));
                 nonfinite = ctx->red_host[2 * k + 3];
             } else {
