@@ -208,14 +208,13 @@ static int precond_into(qxd_ctx* ctx, int fl, int Pv, int Pb, int kind, const vo
     return blas_axpby(ctx, Pv, Pb, n, 1.0, 0.0, ztmp, 0.0, 0.0, z, st);
 }
 
-// Restarted minimal residuals without a preconditioner in FP32, restart lengths up to 16: in
+// Restarted minimal residuals without a preconditioner in FP32, restart lengths up to 8: in
 // exact arithmetic the iterates of GCR(nkv), from a basis that needs no vector update.
 //
 // A cycle forms z_0 = r, z_{k+1} = (Dhat - d) z_k / u_k with the inner products <z_j, z_{k+1}> from
-// the operator's second launch (from the ninth step on those with z_0 .. z_{k-9} in a pass of
-// their own), so that the Gram matrix G of z_0 .. z_K is known.  The u_k are powers of two (exact)
-// that keep |z_k| near |r|: |Dhat - d| to the sixteenth power is 1e9 and more, and FP32 sums of
-// squares would overflow for sources of width 1e11.  With
+// the operator's second launch, so that the Gram matrix G of z_0 .. z_K is known.  The u_k are
+// powers of two (exact) that keep |z_k| near |r|: otherwise |z_8| is 3e4 |r| and FP32 sums of
+// squares overflow for sources of width 2e15.  With
 // a_k = Dhat z_k = u_k z_{k+1} + d_k z_k the correction sum_k c_k z_k of minimal residual solves
 // M c = <a, r>, M = (<a_i, a_k>), by a Cholesky factorisation that grows by one row per
 // step; its forward substitution gives the residual norm after every step.  d is the
@@ -226,9 +225,14 @@ static int precond_into(qxd_ctx* ctx, int fl, int Pv, int Pb, int kind, const vo
 // Why: orthogonalising w_k and updating r in a pass of its own (k_gcr_update, (k + 4) fields)
 // was 16 % of the solve on 32^3x64 C*, and the host looked at every step's numbers before the
 // next was launched.  Solve to 1e-10 there (nkv 8) 72.8 -> 59.7 ms, 56 iterations both; the
-// pivots stay above 1e-5.  From 17 on the powers would end most cycles early: GCR is kept.
-constexpr int kPowerMax = 16;
-static_assert(kPowerMax <= 2 * kMultiMax && kPowerMax * kPowerMax + 5 * kPowerMax + 4 <= kRedSlots, "results of a cycle");
+// pivots stay above 1e-5.  Longer cycles lose the precision of the inner products: with nkv 12
+// and 16 (4 x 4 x 6 x 8 and 8^4, kappa 0.126 and 0.134) the residual norm that the recursion
+// gives fell below the target, or below zero, while the true one was 15 times it, and a third
+// outer step was needed (81 iterations where GCR(16) takes 72).  Ending them early instead
+// costs iterations (16^4, kappa 0.134, nkv 16: 363 where GCR and its fallback take 164).  So from
+// 9 on GCR is kept (24^3 x 12, kappa 0.126, nkv 16: 12.6 ms; by such powers 9.6 ms).
+constexpr int kPowerMax = kMultiMax;
+static_assert(kPowerMax * kPowerMax + 5 * kPowerMax + 4 <= kRedSlots, "results of a cycle");
 
 static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b, void* e, int max_iter, double rtol,
                        int* iters, bool* stagnated, cudaStream_t st) {
@@ -277,10 +281,7 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
         double size = 0.5 * std::log2(std::max(G[K * m + K].real() / G[0].real(), 1e-30)) + growth;  // of |z_{k+1}|
         for (int i = K; i < k; ++i) size += growth - std::log2(u[i]);
         u[k] = std::exp2(std::round(std::min(std::max(size, -60.0), 60.0)));
-        const int rest = std::max(0, k - kMultiMax);
-        QXD_TRY(op_Dhat_dots(ctx, fl, z[k], const_cast<void*>(z[k + 1]), to, k - rest, z.data() + rest, shift,
-                             1.0 / u[k], slot + 2 * rest, st));
-        if (rest > 0) QXD_TRY(blas_multi_dot(ctx, QXD_FP32, n, rest, z.data(), z[k + 1], slot, st));
+        QXD_TRY(op_Dhat_dots(ctx, fl, z[k], const_cast<void*>(z[k + 1]), to, k, z.data(), shift, 1.0 / u[k], slot, st));
         QXD_CUDA(ctx, cudaMemcpyAsync(ctx->red_host + slot, ctx->red_result + slot, sizeof(double) * (2 * k + 4),
                                       cudaMemcpyDeviceToHost, st));
         QXD_CUDA(ctx, cudaEventRecord(ev.e[k & 1], st));
