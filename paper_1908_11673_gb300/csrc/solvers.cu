@@ -219,8 +219,19 @@ static int precond_into(qxd_ctx* ctx, int fl, int Pv, int Pb, int kind, const vo
 // M c = <a, r>, M = (<a_i, a_k>), by a Cholesky factorisation that grows by one row per
 // step; its forward substitution gives the residual norm after every step.  d is the
 // Rayleigh quotient of the first residual: it centres the spectrum, so that the powers stay
-// apart.  A pivot below 1e-7 of its diagonal (the basis is used up at the precision of the
-// sums) ends the cycle there.  The restart takes r = b - Dhat e anew.
+// apart.  The restart takes r = b - Dhat e anew.
+//
+// Precision.  A pivot is the square of a_k - sum_i g_i a_i and comes from sums of FP32 products: with
+// s_k^2 = |u_k z_{k+1}|^2 + |d z_k|^2 and S_k = s_k + sum_i |g_i| s_i their rounding is up to 5e-9 S_k^2
+// of it (768 even sites, against FP64 products of the same fields; less on larger lattices).  A
+// pivot below 1e-8 S_k^2 ends the cycle: the basis is used up.  A residual norm that is 1e-3 of the
+// cycle's first or less is formed anew before it counts.  A cycle that ends before three quarters
+// of its steps, or by either limit without halving the residual norm, says that powers are no basis
+// for this operator and residual (few distinct eigenvalues, a residual of small ones), not that
+// restarted GCR stalls: *lost is set, with |r|^2 and |b|^2, and the caller goes on with GCR steps from
+// e and r.  A limit of 1e-7 of the diagonal instead, and none on the norm, left a residual of 3.6 |b|
+// on the free field 4^4 with bare mass 5e-4 and took such a basis for a stall.  On interacting
+// fields (kappa 0.126 to 0.1355, 8^4 to 32 x 32 x 16 x 16) the iterations with nkv 8 are those of GCR.
 //
 // Why: orthogonalising w_k and updating r in a pass of its own (k_gcr_update, (k + 4) fields)
 // was 16 % of the solve on 32^3x64 C*, and the host looked at every step's numbers before the
@@ -235,7 +246,7 @@ constexpr int kPowerMax = kMultiMax;
 static_assert(kPowerMax * kPowerMax + 5 * kPowerMax + 4 <= kRedSlots, "results of a cycle");
 
 static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b, void* e, int max_iter, double rtol,
-                       int* iters, bool* stagnated, cudaStream_t st) {
+                       int* iters, bool* stagnated, bool* lost, double* rr_out, double* bb_out, cudaStream_t st) {
     using C = std::complex<double>;
     const int nkv = std::max(1, s->nkv);
     const size_t n = 12ull * ctx->g.Vh;
@@ -250,6 +261,7 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
     QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "GCR source"));
     double rr = ctx->red_host[0];
     const double target = rtol * rtol * rr;
+    *bb_out = rr;
     *iters = 0;
     if (rr == 0.0) return QXD_OK;
     std::vector<const void*> z(nkv + 1);
@@ -269,7 +281,8 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
     } ev{st};
     for (auto& x : ev.e) QXD_CUDA(ctx, cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
     const int m = nkv + 1;
-    std::vector<C> G(m * m), L(nkv * nkv), y(nkv), c(nkv);
+    std::vector<C> G(m * m), L(nkv * nkv), y(nkv), c(nkv), g(nkv);
+    std::vector<double> size(nkv);
     std::vector<double> d(nkv, 0.0), u(nkv, 1.0);  // z_{k+1} = (Dhat - d_k) z_k / u_k
     double shift = 0.0;  // an FP32 number, as the kernel applies it
     double growth = 0.0;  // log2 of |(Dhat - d) z_k| / |z_k|, the last one known
@@ -278,9 +291,9 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
     auto launch = [&](int k, int K) -> int {
         const int slot = k * k + 3 * k;
         d[k] = shift;
-        double size = 0.5 * std::log2(std::max(G[K * m + K].real() / G[0].real(), 1e-30)) + growth;  // of |z_{k+1}|
-        for (int i = K; i < k; ++i) size += growth - std::log2(u[i]);
-        u[k] = std::exp2(std::round(std::min(std::max(size, -60.0), 60.0)));
+        double big = 0.5 * std::log2(std::max(G[K * m + K].real() / G[0].real(), 1e-30)) + growth;  // |z_{k+1}|
+        for (int i = K; i < k; ++i) big += growth - std::log2(u[i]);
+        u[k] = std::exp2(std::round(std::min(std::max(big, -60.0), 60.0)));
         QXD_TRY(op_Dhat_dots(ctx, fl, z[k], const_cast<void*>(z[k + 1]), to, k, z.data(), shift, 1.0 / u[k], slot, st));
         QXD_CUDA(ctx, cudaMemcpyAsync(ctx->red_host + slot, ctx->red_result + slot, sizeof(double) * (2 * k + 4),
                                       cudaMemcpyDeviceToHost, st));
@@ -329,7 +342,14 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
                 continue;
             }
             const double pivot = L[k * nkv + k].real();
-            if (!(pivot > 1e-7 * diag) || !(diag > 1e-6 * scale) || !std::isfinite(pivot)) {
+            double S = size[k] = std::sqrt(scale);
+            for (int i = k - 1; i >= 0; --i) {  // L^+ g = (row k of L)^*
+                g[i] = std::conj(L[k * nkv + i]);
+                for (int q = i + 1; q < k; ++q) g[i] -= std::conj(L[q * nkv + i]) * g[q];
+                g[i] /= L[i * nkv + i];
+                S += std::abs(g[i]) * size[i];
+            }
+            if (!(pivot > 1e-8 * S * S) || !std::isfinite(pivot)) {
                 if (k == 0) return qxd_fail(ctx, QXD_EBREAKDOWN, "GCR: |w| = 0");
                 used_up = true;
                 break;
@@ -363,15 +383,18 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
             cim[k] = c[k].imag();
         }
         if (K > 0) QXD_TRY(blas_multi_axpy(ctx, QXD_FP32, QXD_FP32, n, K, cre, cim, z.data(), e, st));
-        ev.ok = reached || *iters >= max_iter;
+        ev.ok = (reached && rr > 1e-6 * rr_cycle) || *iters >= max_iter;
         if (ev.ok) return QXD_OK;
         QXD_TRY(op_Dhat_resid(ctx, fl, b, e, r, to, 0, st));
         QXD_TRY(blas_fetch(ctx, 2, st));
         QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "GCR"));
         rr = ctx->red_host[0];
         // a whole cycle that did not halve the residual norm: restarted GCR stalls
-        *stagnated = rr > target && (K == nkv || used_up) && rr > 0.25 * rr_cycle;
-        ev.ok = rr <= target || *stagnated;
+        const bool slow = rr > 0.25 * rr_cycle;
+        *lost = rr > target && ((used_up && 4 * K < 3 * nkv) || ((used_up || reached) && slow));
+        *stagnated = rr > target && !*lost && K == nkv && slow;
+        *rr_out = rr;
+        ev.ok = rr <= target || *stagnated || *lost;
         if (ev.ok) return QXD_OK;
         z[0] = r;
     }
@@ -379,11 +402,18 @@ static int gcr_power32(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* b,
     return QXD_OK;
 }
 
-int fgcr_inner(qxd_ctx* ctx, int fl, int P, const qxd_solver* s, const void* b, void* e, int max_iter,
-               double rtol, int* iters, bool* stagnated, cudaStream_t st) {
+// *powers: the power basis may be used; cleared for the solves after the one that lost it
+static int fgcr_inner(qxd_ctx* ctx, int fl, int P, const qxd_solver* s, const void* b, void* e, int max_iter,
+                      double rtol, int* iters, bool* stagnated, bool* powers, cudaStream_t st) {
     *stagnated = false;
-    if (P == QXD_FP32 && s->precond == QXD_PRECOND_NONE && s->nkv <= kPowerMax)
-        return gcr_power32(ctx, fl, s, b, e, max_iter, rtol, iters, stagnated, st);
+    *iters = 0;
+    bool go_on = false;  // from the e and r that the power basis leaves
+    double rr = 0.0, bb = 0.0;
+    if (*powers && P == QXD_FP32 && s->precond == QXD_PRECOND_NONE && s->nkv <= kPowerMax) {
+        QXD_TRY(gcr_power32(ctx, fl, s, b, e, max_iter, rtol, iters, stagnated, &go_on, &rr, &bb, st));
+        if (!go_on) return QXD_OK;
+        *powers = false;
+    }
     const int Pb = P, Pv = vec_prec(P);
     const bool split = Pb != Pv;
     const int nkv = s->nkv < 1 ? 1 : (s->nkv > 64 ? 64 : s->nkv);
@@ -404,15 +434,16 @@ int fgcr_inner(qxd_ctx* ctx, int fl, int P, const qxd_solver* s, const void* b, 
         Z[k] = static_cast<char*>(Zb) + (size_t)k * hbb;
         W[k] = static_cast<char*>(Wb) + (size_t)k * hbb;
     }
-    QXD_CUDA(ctx, cudaMemsetAsync(e, 0, hv, st));
-    QXD_CUDA(ctx, cudaMemcpyAsync(r, b, hv, cudaMemcpyDeviceToDevice, st));
-    QXD_TRY(blas_norm2(ctx, Pv, n, b, 0, st));
-    QXD_TRY(blas_fetch(ctx, 2, st));
-    QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "GCR source"));
-    const double bn = std::sqrt(ctx->red_host[0]);
-    *iters = 0;
+    if (!go_on) {
+        QXD_CUDA(ctx, cudaMemsetAsync(e, 0, hv, st));
+        QXD_CUDA(ctx, cudaMemcpyAsync(r, b, hv, cudaMemcpyDeviceToDevice, st));
+        QXD_TRY(blas_norm2(ctx, Pv, n, b, 0, st));
+        QXD_TRY(blas_fetch(ctx, 2, st));
+        QXD_TRY(status_of_norm(ctx, ctx->red_host[1], "GCR source"));
+        rr = bb = ctx->red_host[0];
+    }
+    const double bn = std::sqrt(bb);
     if (bn == 0.0) return QXD_OK;
-    double rr = bn * bn;
     std::vector<double> Rre(nkv * nkv), Rim(nkv * nkv), are(nkv), aim(nkv), ww(nkv), cre(nkv), cim(nkv);
     std::vector<const void*> Wc(nkv + 1);
     bool done = false;
@@ -642,7 +673,7 @@ int solve_fgcr_dc(qxd_ctx* ctx, int fl, const qxd_solver* s, const Full& eta, co
         return QXD_OK;
     };
     double relres = 1.0;
-    bool use_cgnr = false;
+    bool use_cgnr = false, powers = true;
     const double itol = s->inner_tol > 0 ? s->inner_tol : (P == QXD_BF16 ? 5e-3 : (P == QXD_FP32 ? 1e-5 : 1e-10));
     for (int outer = 0; outer < 64; ++outer) {
         if (outer > 0) {
@@ -664,7 +695,7 @@ int solve_fgcr_dc(qxd_ctx* ctx, int fl, const qxd_solver* s, const Full& eta, co
         const double rtol = std::max(itol, 0.5 * s->tol / relres);
         if (!use_cgnr) {
             bool stag = false;
-            QXD_TRY(fgcr_inner(ctx, fl, P, s, bP, eeP, s->nmx - info->iters, rtol, &it, &stag, st));
+            QXD_TRY(fgcr_inner(ctx, fl, P, s, bP, eeP, s->nmx - info->iters, rtol, &it, &stag, &powers, st));
             info->iters += it;
             info->op_applies += it + 2;
             if (stag) {

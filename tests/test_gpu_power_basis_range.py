@@ -1,10 +1,12 @@
 """Unpreconditioned FP32 inner solves at the ends of the power basis: sources far from 1 in
-size, and the tolerance of the inner solves."""
+size, and operators and sources whose powers are no basis."""
 import numpy as np
 import pytest
 
+from oracle import DiracOperator, Flavour, GaugeField, Geometry
+from oracle.solvers import gcr
 from paper_1908_11673_gb300 import workload
-from tests.gpu_helpers import setup
+from tests.gpu_helpers import need_gpu, setup
 
 pytestmark = pytest.mark.gpu
 
@@ -37,4 +39,41 @@ def test_inner_solves_reach_their_tolerance(L, kappa, stout, nkv):
     assert np.linalg.norm(b) < np.linalg.norm(eta)
     assert info.restarts == 1
     assert np.linalg.norm(eta - op.apply(psi)) <= 1e-10 * np.linalg.norm(eta)
+    ctx.close()
+
+
+@pytest.mark.parametrize("L,m0,nkv", [((4, 4, 4, 4), 5e-4, 8), ((4, 4, 4, 4), 5e-4, 16), ((8, 4, 4, 4), 5e-3, 16)])
+def test_powers_of_few_eigenvalues(L, m0, nkv):
+    # Free field, bare mass m0: Dhat has a few distinct eigenvalues, about 2 m0 on constant spinors.
+    # The powers of a source that is mostly constant are parallel to FP32 precision after a few
+    # steps, while the steps of GCR go on reducing the residual.
+    kappa = 0.5 / (4 + m0)
+    zero = (0.0, 0.0, 0.0, 0.0)
+    qxd = need_gpu()
+    geom = Geometry(L, 0, zero)
+    U = np.broadcast_to(np.eye(3, dtype=complex), (geom.V, 4, 3, 3)).copy()
+    A = np.zeros((geom.V, 4))
+    op = DiracOperator(GaugeField(geom, U, A, 6.0), Flavour(4, kappa, 1.0, 1.0))
+    ctx = qxd.Context(L, 0, zero)
+    ctx.set_links(U, A, 6.0)
+    ctx.set_clover(0, 4, kappa, 1.0, 1.0)
+    ev = op.even_sites()
+    lo = np.random.default_rng(3).standard_normal((4, 3))
+    b = lo + 0.1 * workload.spinor(geom.V // 2, 5)
+    eta = np.zeros((geom.V, 4, 3), dtype=complex)
+    eta[ev] = b
+    psi = np.empty_like(eta)
+    info = ctx.solve(0, eta, psi, nkv=nkv, inner=qxd.FP32, tol=1e-9)
+    assert np.linalg.norm(eta - op.apply(psi)) <= 1e-9 * np.linalg.norm(eta)
+    # an FP32 solve leaves about 1e-7 times the condition number, 4 / m0, of its source
+    assert info.restarts <= 2
+    if nkv == 16:
+        # GCR to the inner solves' 1e-5 as often, and two cycles for FP32 rounding
+        Dinv = op.Doo_inv()
+        its = 0
+        for _ in range(1 + info.restarts):
+            x, n = gcr(lambda v: op.Dhat(v, Dinv), b, 1e-5, nkv, 1000)
+            b = b - op.Dhat(x, Dinv)
+            its += n
+        assert info.iters <= its + 2 * nkv
     ctx.close()
