@@ -170,7 +170,8 @@ int qxd_set_links(qxd_ctx* ctx, const double* U, const double* A, double invqel,
 /* Build, for flavour slot fl (0..7), the hopping phases z^qhat (with the
  * boundary phases folded in), the site-diagonal term 1/(2 kappa) + dD_sw + dD_b
  * (eq. sw-term; two Hermitian 6x6 chiral blocks per site) and its inverse on
- * every site, in FP64 with FP32 and BF16 copies.
+ * every site, in FP64 with FP32 and BF16 copies.  Keeps a workspace of up to 512 MB,
+ * which is given back when the context runs short of memory.
  * Errors: QXD_ESTATE before qxd_set_links; QXD_EARG for fl outside 0..7 or
  * kappa <= 0; QXD_ENAN if a diagonal block is singular.  Synchronises `stream`. */
 int qxd_set_clover(qxd_ctx* ctx, int fl, const qxd_flavour* f, void* stream);
@@ -204,7 +205,9 @@ int qxd_solve(qxd_ctx* ctx, int fl, const qxd_solver* s, const void* eta, void* 
  * for j = 0..nshift-1 (1 <= nshift <= 32, sigma[j] >= 0), phi_e and each x_j
  * complex128 [V/2][4][3]; x_e holds the nshift solutions one after the other.
  * s->inner = QXD_FP64 runs the Krylov space in FP64; QXD_FP32 runs it with the
- * FP32 operator and then refines each shift by FP64 defect correction. */
+ * FP32 operator and then refines each shift by FP64 defect correction, the shifts
+ * together: six FP32 even-site fields per shift, at most 2 GB each, are kept for the
+ * next call and given back when the context runs short of memory. */
 int qxd_solve_multishift(qxd_ctx* ctx, int fl, int nshift, const double* sigma, const qxd_solver* s,
                          const void* phi_e, void* x_e, qxd_info* info, void* stream);
 

@@ -28,34 +28,41 @@ int qxd_fail(qxd_ctx* ctx, int code, const std::string& msg) {
     return code;
 }
 
-// Device memory of `bytes` bytes; when there is none left, the field buffers that
-// qxd_set_links kept for flavours not set again since and the SAP copies (the sweeps do
-// without) are given back first.
-bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes) {
-    const cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaSuccess) return true;
-    cudaGetLastError();
-    *p = nullptr;
-    if (e != cudaErrorMemoryAllocation) return false;
-    for (auto& F : ctx->fl) {
-        if (!F.set && !F.building) free_fields(F);
-        if (F.sap) {
-            cudaFree(F.sap);
-            F.sap = nullptr;
-            F.sap_off = true;
-        }
-    }
-    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
-    cudaGetLastError();
-    *p = nullptr;
-    return false;
-}
-
 void qxd_ws_free(qxd_ctx* ctx, int slot) {
     if (slot < 0 || slot >= (int)ctx->ws_ptr.size()) return;
     cudaFree(ctx->ws_ptr[slot]);
     ctx->ws_ptr[slot] = nullptr;
     ctx->ws_size[slot] = 0;
+}
+
+// Device memory of `bytes` bytes; when there is none left, what the context keeps and can do
+// without is given back: first large workspaces that hold nothing between calls (the clover
+// leaves, the corrections of the multi-shift solver), then the field buffers that qxd_set_links kept
+// for flavours not set again since and the SAP copies (the sweeps then read the fields).
+bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes) {
+    for (int stage = 0;; ++stage) {
+        const cudaError_t e = cudaMalloc(p, bytes);
+        if (e == cudaSuccess) return true;
+        cudaGetLastError();
+        *p = nullptr;
+        if (e != cudaErrorMemoryAllocation || stage == 2) return false;
+        if (stage == 0) {
+            bool building = false;
+            for (const auto& F : ctx->fl) building = building || F.building;
+            if (!building) qxd_ws_free(ctx, WS_CLOVER);
+            if (!ctx->refining)
+                for (int k : kRefineSlots) qxd_ws_free(ctx, WS_SOLVER + k);
+        } else {
+            for (auto& F : ctx->fl) {
+                if (!F.set && !F.building) free_fields(F);
+                if (F.sap) {
+                    cudaFree(F.sap);
+                    F.sap = nullptr;
+                    F.sap_off = true;
+                }
+            }
+        }
+    }
 }
 
 int qxd_ws(qxd_ctx* ctx, int slot, size_t bytes, void** out) {

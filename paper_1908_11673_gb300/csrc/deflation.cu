@@ -857,12 +857,12 @@ int qxd_dfl_setup(qxd_ctx* ctx, int fl, const qxd_dfl_params* prm, const void* s
     const size_t fs = field_chunks(ctx);
     const int Ns = prm->Ns;
     if (!dev_alloc(ctx, reinterpret_cast<void**>(&F.dfl_basis), sizeof(float4) * fs * Ns) ||
-        !dev_alloc(ctx, reinterpret_cast<void**>(&F.dfl_A), sizeof(float2) * (size_t)G.Nb * 9 * Ns * Ns)) {
+        !dev_alloc(ctx, reinterpret_cast<void**>(&F.dfl_A), sizeof(float2) * (size_t)G.Nb * 9 * Ns * Ns) ||
+        !dev_alloc(ctx, reinterpret_cast<void**>(&F.dfl_nbr), sizeof(int) * (size_t)G.Nb * 9) ||
+        !dev_alloc(ctx, reinterpret_cast<void**>(&F.dfl_stat), sizeof(CgStat))) {
         dfl_free(F);
         return qxd_fail(ctx, QXD_ECUDA, "dfl_setup: cudaMalloc failed");
     }
-    QXD_CUDA(ctx, cudaMalloc(&F.dfl_nbr, sizeof(int) * (size_t)G.Nb * 9));
-    QXD_CUDA(ctx, cudaMalloc(&F.dfl_stat, sizeof(CgStat)));
     QXD_CUDA(ctx, cudaMemsetAsync(F.dfl_stat, 0, sizeof(CgStat), st));
     F.dfl_Ns = Ns;
     F.dfl_ctol = prm->ctol;

@@ -1175,10 +1175,8 @@ int qxd_set_precond_weights(qxd_ctx* ctx, int fl, const float* W, int nlayers, i
     const size_t nw = ptc_weight_count(nlayers, nch);
     cudaFree(F.W);
     F.W = nullptr;
-    if (cudaMalloc(&F.W, nw * sizeof(float2)) != cudaSuccess) {
-        cudaGetLastError();
+    if (!dev_alloc(ctx, &F.W, nw * sizeof(float2)))
         return qxd_fail(ctx, QXD_ENOMEM, "set_precond_weights: allocation failed");
-    }
     QXD_CUDA(ctx, cudaMemcpy(F.W, W, nw * sizeof(float2), cudaMemcpyDefault));
     F.nlayers = nlayers;
     F.nch = nch;

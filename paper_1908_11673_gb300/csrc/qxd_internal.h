@@ -51,6 +51,7 @@ struct qxd_ctx {
     // workspace: named device buffers, grown on demand, freed in qxd_destroy
     std::vector<void*> ws_ptr;
     std::vector<size_t> ws_size;
+    bool refining = false;  // inside solve_mscg's corrections: kRefineSlots are in use
     double* red_partials = nullptr;  // reduction scratch (per-block partial sums)
     double* red_result = nullptr;    // reduction results (device)
     unsigned* red_ticket = nullptr;  // last-block ticket of the reductions (0 between launches)
@@ -140,6 +141,9 @@ enum {
     WS_CLOVER = 318,
     WS_NSLOTS = 320
 };
+
+// the multi-shift solver's corrections (solve_mscg): slots behind WS_SOLVER
+constexpr int kRefineSlots[] = {115, 116, 117, 118, 120, 121};
 
 // kernels launched from other translation units ------------------------------------
 namespace qxd {

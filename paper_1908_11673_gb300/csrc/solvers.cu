@@ -1076,16 +1076,20 @@ int solve_mscg(qxd_ctx* ctx, int fl, int ns, const double* sigma, const qxd_solv
     // on large lattices
     const size_t h32 = half_bytes(ctx, QXD_FP32);
     int group = (int)std::max<size_t>(1, std::min<size_t>(ns, kRefineBytes / h32));
+    struct Refining {  // until the return the fields are not spare (dev_alloc)
+        qxd_ctx* ctx;
+        explicit Refining(qxd_ctx* c) : ctx(c) { ctx->refining = true; }
+        ~Refining() { ctx->refining = false; }
+    } in_use(ctx);
     CgFields work{};
     void *rb, *eb;
+    void** const fields[] = {&work.r, &work.p, &work.w, &work.t, &eb, &rb};  // in kRefineSlots
     for (;; group = (group + 1) / 2) {  // fewer at a time where there is no memory for them
-        const std::pair<int, void**> fields[] = {{121, &rb}, {120, &eb}, {115, &work.r}, {116, &work.p}, {117, &work.w}, {118, &work.t}};
         int rc = QXD_OK;
-        for (const auto& f : fields)
-            if (rc == QXD_OK) rc = qxd_ws(ctx, WS_SOLVER + f.first, h32 * group, f.second);
+        for (int k = 0; k < 6 && rc == QXD_OK; ++k) rc = qxd_ws(ctx, WS_SOLVER + kRefineSlots[k], h32 * group, fields[k]);
         if (rc == QXD_OK) break;
         if (group == 1) return rc;
-        for (const auto& f : fields) qxd_ws_free(ctx, WS_SOLVER + f.first);
+        for (int k : kRefineSlots) qxd_ws_free(ctx, WS_SOLVER + k);
     }
     double worst = 0.0;
     for (int j0 = 0; j0 < ns; j0 += group) {
