@@ -319,7 +319,8 @@ int qxd_set_precond_weights(qxd_ctx* ctx, int fl, const float* W, int nlayers, i
  * block at the start of its colour's sweep.  FGCR on Dhat uses z_e = (M (r_e, 0))_e (Dhat^-1 = (D^-1)_ee).
  * Arithmetic in FP32.  The first sweep after qxd_set_clover lays the links and
  * site-diagonal terms out by block (720 bytes of device memory per site and flavour
- * slot, given back when the context runs short of memory; not under stream capture). */
+ * slot, kept for later terms and given back when the context runs short of memory; not
+ * under stream capture). */
 
 /* Set ncy and nmr (1..64 each; default 5 and 5, the paper's values). */
 int qxd_set_sap(qxd_ctx* ctx, int ncy, int nmr);

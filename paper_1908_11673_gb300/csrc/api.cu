@@ -58,6 +58,7 @@ bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes) {
                 if (F.sap) {
                     cudaFree(F.sap);
                     F.sap = nullptr;
+                    F.sap_built = false;
                     F.sap_off = true;
                 }
             }
@@ -203,12 +204,12 @@ bool make_geo(const qxd_geom* g, Geo* G) {
     return true;
 }
 
-// drops everything a flavour holds but its field buffers, which qxd_set_clover fills again
+// drops everything a flavour holds but the buffers that are filled again: of its fields by
+// qxd_set_clover, of the SAP copies by the next sweep
 static void reset_flavour(QxdFlavour& F) {
     cudaFree(F.Cdf[0]);
     cudaFree(F.Cdf[1]);
     cudaFree(F.Vdf);
-    cudaFree(F.sap);
     cudaFree(F.W);
     cudaFree(F.dfl_basis);
     cudaFree(F.dfl_A);
@@ -217,6 +218,7 @@ static void reset_flavour(QxdFlavour& F) {
     QxdFlavour kept{};
     kept.V64 = F.V64;
     kept.Z32 = F.Z32;
+    kept.sap = F.sap;
     for (int k = 0; k < 2; ++k) {
         kept.C64[k] = F.C64[k];
         kept.C32[k] = F.C32[k];
@@ -227,6 +229,8 @@ static void reset_flavour(QxdFlavour& F) {
 static void free_flavour(QxdFlavour& F) {
     reset_flavour(F);
     free_fields(F);
+    cudaFree(F.sap);
+    F.sap = nullptr;
 }
 
 extern "C" {
@@ -330,14 +334,14 @@ int qxd_set_clover(qxd_ctx* ctx, int fl, const qxd_flavour* f, void* stream) {
         }
     }
     F.f = *f;
-    // double-float and SAP copies and a deflation subspace belong to the operator they were built for
+    // double-float and SAP copies and a deflation subspace belong to the operator they were built
+    // for (the buffer of the SAP copies is filled again by the next sweep)
     cudaFree(F.Vdf);
     cudaFree(F.Cdf[0]);
     cudaFree(F.Cdf[1]);
     F.Vdf = nullptr;
     F.Cdf[0] = F.Cdf[1] = nullptr;
-    cudaFree(F.sap);
-    F.sap = nullptr;
+    F.sap_built = false;
     F.sap_off = false;
     dfl_free(F);
     const int rc = launch_set_flavour(ctx, fl, st);

@@ -24,6 +24,7 @@ struct QxdFlavour {
     float4* Vdf = nullptr;                 // [p][36][Vh]  V64 as double-float pairs (on first use)
     float4* Cdf[2] = {nullptr, nullptr};   // [p][36][Vh]  C64[0] as double-float pairs (on first use; [1] unused)
     void* sap = nullptr;       // SAP: the blocks' own copies of links and terms (on first use)
+    bool sap_built = false;    // they are those of the present links and terms
     bool sap_off = false;      // no memory for them
     // learned preconditioner
     void* W = nullptr;         // device weights (complex float [layers][cout][cin][9][4][4])

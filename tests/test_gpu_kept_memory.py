@@ -36,3 +36,38 @@ def test_workspaces_that_hold_nothing_are_given_back(shifts, Ns):
     ctx.dfl_basis(0, 0, out)
     assert abs(float(torch.linalg.vector_norm(out)) - np.sqrt(V / 256)) < 1e-3  # norm 1 on every block
     ctx.close()
+
+
+def test_sap_copies_keep_their_buffer(monkeypatch):
+    # a new term or a new gauge field fills the buffer again: nothing is freed and allocated for it
+    import torch
+    L = (16, 16, 16, 16)
+    qxd, ctx, op, _, _ = setup(L, 0, PI, kappa=0.126, device="cuda")
+    U, A = (torch.from_numpy(f).cuda() for f in workload.gauge_field(L, 2000, device="cuda"))
+    ctx.set_sap(1, 2)
+    eta = torch.randn(op.geom.V, 4, 3, dtype=torch.complex64, device="cuda")
+    copies, fields = torch.empty_like(eta), torch.empty_like(eta)
+
+    def used():
+        torch.cuda.synchronize()
+        free, total = torch.cuda.mem_get_info()
+        return total - free
+
+    def sweep():
+        ctx.sap_apply(0, eta, copies)
+        with monkeypatch.context() as m:
+            m.setenv("QXD_SAP_BLOCKS", "0")
+            ctx.sap_apply(0, eta, fields)
+        assert torch.equal(copies, fields)
+
+    sweep()
+    held = used()
+    ctx.set_clover(0, -2, 0.12, 1.9, 1.0)
+    assert used() == held
+    sweep()
+    ctx.set_links(U, A)
+    ctx.set_clover(0, -2, 0.12, 1.9, 1.0)
+    assert used() == held
+    sweep()
+    assert used() == held
+    ctx.close()
