@@ -450,8 +450,11 @@ __global__ void __launch_bounds__(kQuadThreads) k_hop_quad(Geo g, CanonDev a, in
     }
 }
 
-// site and right-hand-side products up to which four lanes per site are the faster
-constexpr long long quad_sites(int prec) { return prec == QXD_FP64 ? 4096 : 8192; }
+// site and right-hand-side products up to which four lanes per site are the faster.  One thread
+// and four lanes (us), by sites of the output times right-hand sides: Dhat FP32 12.3 and 6.3 at 4096,
+// 11.5 at 8192, FP64 83.9 and 44 at 2048, 76 at 4096; D_w FP32 6.1 and 4.1 at 7168, 4.2 to 7.5 at
+// 8192, 9.4 at 10240, FP64 40.9 and 15.6 at 2560, 42.4 at 3072, 48.5 at 4096
+constexpr long long quad_sites(int prec, int mode) { return prec != QXD_FP64 ? 8192 : mode == kDw ? 2560 : 4096; }
 
 template <int P, int MODE>
 cudaError_t launch_quad(const Geo& g, const CanonDev& a, int nrhs, cudaStream_t st) {
@@ -488,7 +491,7 @@ int launch_canon(qxd_ctx* ctx, int fl, int prec, const void* nb, const void* sel
     for (int k = 0; k < parts; ++k) {
         const int first = k * (sites / parts), end = k + 1 == parts ? sites : (k + 1) * (sites / parts);
         ProfScope prof(ctx, name, (double)g.Vh * ((MODE == kDw ? link + 2 * dg : link + dg) + per * nrhs) / parts, st);
-        if (prec != QXD_BF16 && (long long)sites * nrhs <= quad_sites(prec)) {
+        if (prec != QXD_BF16 && (long long)sites * nrhs <= quad_sites(prec, MODE)) {
             const cudaError_t e = prec == QXD_FP64 ? launch_quad<0, MODE>(g, a, nrhs, st) : launch_quad<1, MODE>(g, a, nrhs, st);
             QXD_CUDA(ctx, e);
             continue;
