@@ -486,7 +486,7 @@ def batched_row(qxd, torch, dev, stream, timed):
     for nrhs in (1, 4, 12):
         x = torch.randn((nrhs, V, 4, 3), dtype=torch.complex64, device=dev, generator=gen)
         y = torch.empty_like(x)
-        ctx.apply_Dw(0, qxd.FP32, x, y, nrhs=nrhs, stream=stream)  # tunes the launch shape
+        ctx.apply_Dw(0, qxd.FP32, x, y, nrhs=nrhs, stream=stream)  # warm-up
         torch.cuda.synchronize()
         ctx.profile(2)
         calls = 10

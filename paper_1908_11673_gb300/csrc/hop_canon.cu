@@ -9,8 +9,9 @@
 //
 // A site's twelve complex numbers are contiguous (96 or 192 bytes, whole 32-byte
 // sectors), so a spinor is three or six 256-bit accesses per thread; links and
-// site-diagonal terms keep the internal layout.  The arithmetic is that of the internal
-// kernels, in the same order.
+// site-diagonal terms keep the internal layout.  k_hop_canon does the arithmetic of the
+// internal kernels in the same order; k_hop_quad, on small lattices, adds the directions in
+// another order.
 //
 // Why: the conversion passes move four spinors per site and right-hand side (384 bytes in
 // FP32, more than the operator itself with many right-hand sides) and cost two to four
@@ -485,7 +486,9 @@ int launch_canon(qxd_ctx* ctx, int fl, int prec, const void* nb, const void* sel
     std::snprintf(name, sizeof name, "hop_%s_%s%s", prec == QXD_FP64 ? "fp64" : prec == QXD_FP32 ? "fp32" : "bf16", mode,
                   nrhs > 1 ? "_mrhs" : "");
     // D_w of several right-hand sides on a large lattice goes over the sites in two launches
-    // (the first and the second half), as many as the half-lattice kernels take
+    // (the first and the second half): as many as over two half lattices, which profiles of
+    // launches count on.  It is not the faster form (24^3x48 with 12 right-hand sides 762 us, 747 in
+    // one launch); 2^20 keeps it away from small lattices, where a second launch costs more.
     const int sites = MODE == kDw ? (int)g.V : g.Vh;
     const int parts = MODE == kDw && nrhs > 1 && (long long)sites * nrhs > (1 << 20) ? 2 : 1;
     for (int k = 0; k < parts; ++k) {

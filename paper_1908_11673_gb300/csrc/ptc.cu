@@ -161,7 +161,7 @@ struct PtcFwdShared {
 
 // weight planes of a layer cin -> cout (adjoint: of the adjoint of the layer cout -> cin with
 // the weights W, W'[c][c'][d] = W[c'][c][opposite(d)]^+): [group of 8 output channels]
-// [pair q = d cin + c'][Re, Im, -Im][s'][4 (c - c0) + s], zero beyond cout
+// [pair q = d cin + c'][Re, Im][s'][4 (c - c0) + s], zero beyond cout
 constexpr int kPlane = 2 * 4 * 4 * kPtcGroup;  // floats of a pair
 
 __global__ void k_ptc_planes(const float2* __restrict__ W, int cin, int cout, int adjoint, float* __restrict__ P) {
