@@ -164,7 +164,8 @@ void qxd_destroy(qxd_ctx* ctx);
  * depend on it (q Ahat = qhat (i/4) Im sum z_{mu nu}).
  * Invalidates every SW term set before; their device memory is kept for the next
  * qxd_set_clover of the same slots (and given back when the context runs short of
- * memory).  Synchronises `stream`. */
+ * memory).  Synchronises `stream`, and waits for operators that are still queued on
+ * other streams. */
 int qxd_set_links(qxd_ctx* ctx, const double* U, const double* A, double invqel, void* stream);
 
 /* Build, for flavour slot fl (0..7), the hopping phases z^qhat (with the

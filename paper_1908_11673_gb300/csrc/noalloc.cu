@@ -90,6 +90,7 @@ extern "C" int qxd_apply_Dhat_eo_noalloc(qxd_ctx* ctx, int fl, int prec, int dag
     void* to = scratch + kNoallocFieldBytes;
     void* oe = scratch + 2 * kNoallocFieldBytes;
     cudaStream_t st = (cudaStream_t)stream;
+    note_operator(ctx, st);
     const int cprec = prec == QXD_FP64 ? 0 : 1;
     // on the caller's fields as qxd_apply_Dhat_eo does it (8^4 FP32: 24 -> 6 us)
     if (canon_fits(in_e, out_e, (size_t)ctx->g.Vh * 12 * (cprec == 0 ? 16 : 8), true))

@@ -79,6 +79,10 @@ struct qxd_ctx {
     // keyed by (precision, self mode, post mode, nrhs, V/2)
     std::map<std::tuple<int, int, int, int, long long>, std::pair<int, int>> tune_hop;
     cudaStream_t cap_stream = nullptr;  // library stream for CUDA-graph capture
+    // the stream of the operators queued since the links were set (compared, never used), whether
+    // there were several, and whether a graph ever took one, which may run on any
+    cudaStream_t op_stream = nullptr;
+    bool op_queued = false, op_several = false, op_graph = false;
     int sap_ncy = 5, sap_nmr = 5;       // SAP preconditioner parameters (qxd_set_sap)
 };
 
@@ -114,6 +118,9 @@ int qxd_fail(qxd_ctx* ctx, int code, const std::string& msg);
 // workspace slot `slot` with at least `bytes` bytes (device memory)
 int qxd_ws(qxd_ctx* ctx, int slot, size_t bytes, void** out);
 void qxd_ws_free(qxd_ctx* ctx, int slot);
+
+// an operator is about to be queued on st and not waited for (api.cu)
+void note_operator(qxd_ctx* ctx, cudaStream_t st);
 
 // device memory for the context (api.cu); false if there is none
 bool dev_alloc(qxd_ctx* ctx, void** p, size_t bytes);
